@@ -312,7 +312,8 @@ def kernel_name(hqa, plan, prec_name):
     k = plan["kernel"]
     if k == hqa.KERNEL_DENSE:
         if prec_name == "PREC_FP32":
-            return "k_dense_simt<1>"
+            # 256 threads: the CUDA-core form; else the fixed-point slices on the tensor cores
+            return "k_dense_simt<1>" if plan.get("threads", 256) == 256 else "k_dense_f32"
         kseg = 2 if prec_name.endswith("X2") else 1
         f16 = "true" if prec_name.startswith("PREC_FP16") else "false"
         return f"k_dense_md<{plan['replicas_per_block'] // 2},*,{kseg},*,*,{f16},*,*,*>"
@@ -820,7 +821,8 @@ def launches_per_step(hqa, plan, hv, cfg, S, batch, real, count):
     if hv["one_at_a_time"]:
         return count * 3      # per member: MD, readout, energy
     if plan["kernel"] == hqa.KERNEL_DENSE and hv["prec_name"] == "PREC_FP32":
-        md = S + 2            # init, one launch per leapfrog step, output
+        md = (S + 2 if plan.get("threads", 256) == 256   # init, one launch per step, output
+              else 4 * plan.get("chunks", 1))             # init, slices, persistent MD, output
     elif plan["kernel"] == hqa.KERNEL_DENSE:
         md = 3 * plan.get("chunks", 1)   # init, persistent MD, output per chunk
     else:

@@ -101,7 +101,8 @@ void free_ctx_device(hqa_ctx* c)
                     c->d_h_i32,   c->d_sched, c->d_ws,     c->d_state,  c->d_sub,
                     c->d_status,  c->d_Jbf,   c->d_binst,  c->d_bwork, c->d_feat,
                     c->d_tune,    c->d_diag,   c->d_Jcat,  c->d_efx,   c->d_ld,
-                    c->d_ldwork,  c->d_Jh,     c->d_Jhcat, c->d_Jf32,  c->d_ebits};
+                    c->d_ldwork,  c->d_Jh,     c->d_Jhcat, c->d_Jf32,  c->d_ebits,
+                    c->d_Jsl,     c->d_Jscale};
     for (void* p : ptrs)
         if (p) cudaFree(p);
 }
@@ -128,6 +129,7 @@ hqa_status finish_create(hqa_ctx* c, hqa_ctx** out)
         if (std::fabs(v) != 1.f) unit = false;
         if (integer) sum += (int64_t)v;
     }
+    c->j_whole = integer;
     c->has_h = false;
     for (float v : c->h) {
         if (v != 0.f) c->has_h = true;
@@ -307,7 +309,8 @@ hqa_status choose_plan(hqa_ctx* ctx, int32_t R, const hqa_run_opts& opts, const 
 }
 
 // Which dense path a single-context run or field takes: 0 none (the sparse
-// kernels), 1 the tcgen05 GEMM (16-bit precisions), 2 the FP32 CUDA-core GEMM.
+// kernels), 1 the tcgen05 GEMM (16-bit precisions), 2 the FP32 one (runs: slices
+// on the tensor cores, or the CUDA-core GEMM; fields: the CUDA-core GEMM).
 // HQA_KERNEL_DENSE asks for the dense path; AUTO takes it for 16-bit
 // precisions on a dense context, for FP32 only when the couplings are not all
 // +-1 (the sparse kernels need them) or the autotuner chose it.
@@ -713,6 +716,9 @@ static hqa_status run_impl(hqa_ctx* ctx, const hqa_schedule* sched, double dt, i
     if (dense == 1)
         s = hqa_dense_launch_md(ctx, ctx->d_sched, steps, sched->window, replicas, seed, o.init,
                                 o.phi0, o.p0, sched->M, out->phi, out->p, phibar, o.precision, st);
+    else if (dense == 2 && hqa_f32tc_possible(ctx))
+        s = hqa_f32tc_launch_md(ctx, ctx->d_sched, steps, sched->window, replicas, seed, o.init,
+                                o.phi0, o.p0, sched->M, out->phi, out->p, phibar, st);
     else if (dense == 2)
         s = hqa_simt_launch_md(ctx, ctx->d_sched, steps, sched->window, replicas, seed, o.init,
                                o.phi0, o.p0, sched->M, out->phi, out->p, phibar, st);
@@ -849,6 +855,21 @@ hqa_status hqa_plan_query(hqa_ctx* ctx, int32_t replicas, const hqa_run_opts* op
     int dense = 0;
     s = pick_dense(ctx, replicas, o, &dense);
     if (s != HQA_OK) return s;
+    if (dense == 2 && hqa_f32tc_possible(ctx)) {
+        int rb = 0, grid = 0, C = 1;
+        s = hqa_f32tc_plan(ctx, replicas, &rb, &grid, &C);
+        if (s != HQA_OK) return s;
+        out->kernel = HQA_KERNEL_DENSE;
+        out->replicas_per_block = rb;
+        out->blocks = grid;
+        out->threads = 320;         // TMA warp, MMA warp, 8 epilogue warps
+        out->smem_bytes = 0;
+        out->chunks = C;
+        out->pad_ratio = (double)C * grid * 128 * rb / ((double)ctx->N * replicas);
+        out->conflict_ratio = 1.0;
+        out->balance = 1.0;
+        return HQA_OK;
+    }
     if (dense == 2) {
         out->kernel = HQA_KERNEL_DENSE;
         out->replicas_per_block = 128;

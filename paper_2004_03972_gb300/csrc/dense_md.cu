@@ -182,12 +182,12 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode()
     return fn;
 }
 
-// 2-D 16-bit tensor [rows][cols] (BF16, or FP16 when f16; cols contiguous,
-// cols * 2 bytes a multiple of 16), box {64 cols, box_rows}, 128-byte swizzle.
+}  // namespace
+
 // A [rows][cols] 16-bit array; box_cols x box_rows boxes, 128-byte swizzle
 // (MMA operand tiles) or none (row-major staging tiles).
-bool make_tmap16_box(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols,
-                     uint32_t box_cols, uint32_t box_rows, bool swizzle, bool f16)
+bool hqa_dense_tmap16(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols,
+                      uint32_t box_cols, uint32_t box_rows, bool swizzle, bool f16)
 {
     auto enc = get_encode();
     if (!enc) return false;
@@ -202,10 +202,13 @@ bool make_tmap16_box(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t co
     return r == CUDA_SUCCESS;
 }
 
+namespace {
+
+// box {64 cols, box_rows}, 128-byte swizzle
 bool make_tmap16(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows,
                  bool f16)
 {
-    return make_tmap16_box(m, ptr, rows, cols, BK, box_rows, true, f16);
+    return hqa_dense_tmap16(m, ptr, rows, cols, BK, box_rows, true, f16);
 }
 
 template <int BN, int STAGES>
@@ -492,7 +495,7 @@ static hqa_status dense_md_chunk(hqa_ctx* ctx, const StepCoef* d_sched, int64_t 
         return HQA_ERR_CUDA;
     // the epilogue's operand stores: 128 spins x 16 replicas per box, unswizzled
     CUtensorMap tmS;
-    if (!make_tmap16_box(&tmS, a.phib, (uint64_t)2 * Rpad, (uint64_t)kseg * Npad, 128, 16, false, f16))
+    if (!hqa_dense_tmap16(&tmS, a.phib, (uint64_t)2 * Rpad, (uint64_t)kseg * Npad, 128, 16, false, f16))
         return HQA_ERR_CUDA;
     const CUtensorMap& tmA = f16 ? (kseg == 3 ? ctx->tmJh3 : ctx->tmJh)
                                  : (kseg == 3 ? ctx->tmJ3 : ctx->tmJ);

@@ -1,7 +1,9 @@
-// dense_simt.cu -- the plain FP32 dense local field and MD step on the CUDA
-// cores (no tensor cores, no reduced precision).
+// dense_simt.cu -- the FP32 dense local field and MD step on the CUDA cores.
 //
-// It is the FP32 reference form of the dense path: the field of all replicas
+// The one-shot FP32 field of a dense context, and the FP32 MD of contexts the
+// tensor-core form (dense_f32.cu) does not take: more row tiles than SMs
+// (N > 19456), which its one-CTA-per-row-tile grid cannot hold at once, where
+// this form's launches need no co-residency.  The field of all replicas
 // is the product L = J Phi (Methods, "Leapfrog algorithm"), evaluated with
 // FP32 fused multiply-adds, and each leapfrog step is one launch of a tiled
 // SGEMM whose epilogue applies the kick and drift to its tile.

@@ -118,6 +118,7 @@ struct hqa_ctx {
     bool dense_input = false;
     bool integer = false;       // all J and h integral with |J| <= 127, |h| <= 2^20
     bool unit = false;          // all J in {-1, 0, +1}
+    bool j_whole = false;       // all J integral with |J| <= 127, whatever h
     bool has_h = false;
 
     // host copies of the symmetric CSR (diagonal dropped), used to build plans
@@ -213,6 +214,13 @@ struct hqa_ctx {
     // plain FP32 dense path (CUDA cores): J in FP32, [Npad32][Npad32], built on first use
     float* d_Jf32 = nullptr;
     int Npad32 = 0;
+    // FP32 dense path on the tensor cores: BF16 slices of J ([Mpad][3 Mpad], the
+    // first nj used, with a power of two per row), built on first use; whole-numbered J uses d_Jbf instead.
+    // 0: not built yet
+    int f32_nj = 0;
+    void* d_Jsl = nullptr;
+    float* d_Jscale = nullptr;
+    CUtensorMap tmJsl;
     // bit-mask integer energy (readout.cu): word-major nonzero and negative masks, degrees
     void* d_ebits = nullptr;
 };
@@ -295,6 +303,17 @@ hqa_status hqa_dense_launch_md(hqa_ctx* ctx, const StepCoef* d_sched, int64_t S,
                                int32_t R, uint64_t seed, int init, const float* phi0,
                                const float* p0, int M, float* phi_out, float* p_out,
                                float* phibar_out, int prec, cudaStream_t st);
+// tensor map of a 16-bit [rows][cols] array (cols contiguous)
+bool hqa_dense_tmap16(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols,
+                      uint32_t box_cols, uint32_t box_rows, bool swizzle, bool f16);
+// dense_f32.cu: the FP32 dense path on the tensor cores (fixed-point slices)
+bool hqa_f32tc_possible(const hqa_ctx* ctx);
+hqa_status hqa_f32tc_prepare(hqa_ctx* ctx);
+hqa_status hqa_f32tc_plan(hqa_ctx* ctx, int32_t R, int* rb, int* grid, int* chunks);
+hqa_status hqa_f32tc_launch_md(hqa_ctx* ctx, const StepCoef* d_sched, int64_t S, int32_t W,
+                               int32_t R, uint64_t seed, int init, const float* phi0,
+                               const float* p0, int M, float* phi_out, float* p_out,
+                               float* phibar_out, cudaStream_t st);
 // dense_simt.cu: the plain FP32 dense path on the CUDA cores
 bool hqa_simt_possible(const hqa_ctx* ctx);
 hqa_status hqa_simt_prepare(hqa_ctx* ctx);
