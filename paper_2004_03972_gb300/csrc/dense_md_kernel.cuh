@@ -81,6 +81,12 @@ constexpr int kMDThreads = 64 + 32 * kEpiWarps;
 constexpr bool kTmaStore = true;
 constexpr uint32_t kStgBytes = 16 * 128 * 2;   // one staging tile [16 replicas][128 spins]
 
+// One window sum: its only owner adds once per step, so the reduction gives
+// the load-add-store's result (bitwise) without waiting for the load.  K2000 x
+// 4096, 40 steps inside the window: FP16X2 2.82 -> 1.99 ms, BF16 2.36 -> 1.56 ms;
+// outside the window a step is unchanged (43 and 30 us).
+__device__ __forceinline__ void win_add(float* w, float v) { atomicAdd(w, v); }
+
 __device__ __forceinline__ void sts_u16(uint32_t a, uint16_t v)
 {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(v) : "memory");
@@ -533,8 +539,8 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
                                 sts_u16(sb + kStgBytes, (uint16_t)l2);
                                 sts_u16(sb + kStgBytes + 256u, (uint16_t)(l2 >> 16));
                                 if (in_win) {
-                                    a.w[o0] += lo2(fn2);
-                                    a.w[o1] += hi2(fn2);
+                                    win_add(a.w + o0, lo2(fn2));
+                                    win_add(a.w + o1, hi2(fn2));
                                 }
                             }
                         } else if (row_ok) {
@@ -565,7 +571,7 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
                                         nb[ob + 2 * a.Npad] = cvt16<F16>(fs - from16<F16>(hi));
                                     }
                                 }
-                                if (in_win) a.w[o] += fn;
+                                if (in_win) win_add(a.w + o, fn);
                             }
                         } else if constexpr (TS) {
                             // spin rows beyond N keep a zero operand
@@ -637,7 +643,7 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
                                     nb[ob + a.Npad] = hi;
                                     nb[ob + 2 * a.Npad] = cvt16<F16>(fs - from16<F16>(hi));
                                 }
-                                if (in_win) a.w[(size_t)(n0 + col + j) * a.Npad + row] += fn;
+                                if (in_win) win_add(a.w + (size_t)(n0 + col + j) * a.Npad + row, fn);
                             }
                         }
                         // .sync.aligned: every lane of the warp, outside the row_ok branch
@@ -686,7 +692,7 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
                                     nb[ob + a.Npad] = hi;
                                     nb[ob + 2 * a.Npad] = cvt16<F16>(fs - from16<F16>(hi));
                                 }
-                                if (in_win) a.w[o] += fn;
+                                if (in_win) win_add(a.w + o, fn);
                             }
                         }
                         if (more) {
