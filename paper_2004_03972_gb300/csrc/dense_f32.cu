@@ -32,13 +32,15 @@
 // (dense_md_kernel.cuh): a TMA producer warp, an MMA warp, epilogue warps,
 // phi in TMEM, p in global memory, a column-group arrival counter per half;
 // pairs of row tiles share cta_group::2 MMAs where the row tiles pair up and
-// J is one slice.  The producer issues the coupling tiles of the next pass
-// before it waits for the column group, since only phi depends on it.
+// J is one slice.  While the producer waits for the column group it already
+// loads coupling tiles into free stages, since only phi depends on the other
+// CTAs (real N = 500 x 200: 7.3 -> 6.9 us per step; filling the ring before
+// looking at the counter cost K2000 x 1024 17.5 -> 18.5 us).
 //
 // What bounds it: the SM's intake from L2, 28 KB per k-tile of a pair's CTA at
 // about 100 GB/s of the 128 that an SM can take (64 B/clk); the MMAs would need
 // two thirds of the step.  Measured against the CUDA-core form
-// (dense_simt.cu), per step: K2000 +-1 x 1024 replicas 210 -> 18.4 us, real
+// (dense_simt.cu), per step: K2000 +-1 x 1024 replicas 210 -> 17.5 us, real
 // N = 1000 x 512 115 -> 10.6 us; error against FP64 after 40 steps (2-norm, p)
 // 6.9e-7 -> 3.8e-7 and 7.6e-7 -> 4.9e-7.
 #include <cuda.h>
@@ -189,15 +191,17 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
         if (lane == 0) {
             // ---- TMA producer ----
             uint32_t it = 0;
-            // the stage of k-tile `kt` is free: its coupling tiles start
+            auto is_free = [&](uint32_t q) {   // the stage of iteration q, without blocking
+                return q < STAGES ||
+                       tc::mbar_test<PAIR>(empty0 + 8 * (q % STAGES), ((q / STAGES) - 1) & 1);
+            };
+            auto wait_free = [&](uint32_t q) {
+                if (q < STAGES) return true;
+                const uint32_t e = empty0 + 8 * (q % STAGES), ph = ((q / STAGES) - 1) & 1;
+                return PAIR ? tc::mbar_wait_cl(e, ph, abort, kWaitNs) : tc::mbar_wait(e, ph, abort, kWaitNs);
+            };
             auto load_j = [&](uint32_t q, int kt) {
                 const int s = q % STAGES;
-                if (q >= STAGES) {
-                    const uint32_t ph = ((q / STAGES) - 1) & 1;
-                    if (!(PAIR ? tc::mbar_wait_cl(empty0 + 8 * s, ph, abort, kWaitNs)
-                               : tc::mbar_wait(empty0 + 8 * s, ph, abort, kWaitNs)))
-                        return false;
-                }
                 tc::mbar_expect_tx(full0 + 8 * s, STAGE);
 #pragma unroll
                 for (int k = 0; k < KSUB; ++k)
@@ -205,7 +209,6 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                     for (int j = 0; j < NJ; ++j)
                         tc::tma_load_2d(base + s * STAGE + (k * NJ + j) * A_BYTES, &tmJ,
                                         j * a.Npad + (kt * KSUB + k) * BK, m0, full0 + 8 * s);
-                return true;
             };
             auto load_b = [&](uint32_t q, int kt, int brow) {
                 const int s = q % STAGES;
@@ -232,32 +235,35 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
             const int KT = a.KT / KSUB;
             for (int64_t m = 0; m < a.S && !*abort; ++m)
                 for (int hh = 0; hh < HV && !*abort; ++hh) {
-                    const int pre = KT < STAGES ? KT : STAGES;
-                    int kt = 0;
-                    for (; kt < pre; ++kt)
-                        if (!load_j(it + kt, kt)) break;
-                    if (*abort) { it += kt; break; }
+                    // until the column group has finished the last step, coupling
+                    // tiles go into whatever stages are free
+                    int pre = 0;
                     if (m > 0) {
                         const unsigned int* g = a.gbar + HV * nc + hh;
                         const unsigned int target = (unsigned int)(a.Mt * m);
                         const uint64_t t0 = tc::globaltimer();
                         uint32_t spins = 0;
                         while (hqa_dense::ld_acquire(g) < target) {
+                            if (pre < STAGES && pre < KT && is_free(it + pre)) {
+                                load_j(it + pre, pre);
+                                ++pre;
+                            }
                             if ((++spins & 63u) == 0) {
                                 if (*abort || (*gstatus & HQA_DEV_TIMEOUT)) { *abort = 1; break; }
                                 if (tc::globaltimer() - t0 > kWaitNs) { *abort = 1; break; }
                             }
                         }
-                        if (*abort) { it += kt; break; }
+                        if (*abort) { it += pre; break; }
                         tc::fence_proxy_async_global();
                     }
                     const int brow = (int)(m & 1) * a.Rpad + n0 + hh * NC;
-                    for (int k = 0; k < pre; ++k) load_b(it + k, k, brow);
-                    for (; kt < KT; ++kt) {
-                        if (!load_j(it + kt, kt)) break;
-                        load_b(it + kt, kt, brow);
+                    for (int kt = 0; kt < KT; ++kt, ++it) {
+                        if (kt >= pre) {
+                            if (!wait_free(it)) break;
+                            load_j(it, kt);
+                        }
+                        load_b(it, kt, brow);
                     }
-                    it += kt;
                 }
             // drain: every issued copy must land before the CTA can exit
             if (*abort)

@@ -56,6 +56,27 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t a, uint32_t parity)
     return ok != 0;
 }
 
+// Whether phase `parity` is complete, without blocking; CL: cluster-scope
+// acquire, as mbar_wait_cl.
+template <bool CL>
+__device__ __forceinline__ bool mbar_test(uint32_t a, uint32_t parity)
+{
+    uint32_t ok;
+    if constexpr (CL)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(a), "r"(parity) : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(a), "r"(parity) : "memory");
+    return ok != 0;
+}
+
 // Waits for phase `parity` of the mbarrier; gives up (returns false, sets
 // *abort) after `limit_ns` or as soon as *abort is set by another thread.
 __device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile int* abort,
