@@ -3,8 +3,8 @@
 // Readout (Results, "Sorting frozen and ambivalent variables"; HQA section):
 //   s_i = sgn(phibar_i) with sgn(0) = +1; spins ordered by (|phibar_i|, i)
 //   ascending; the first n are ambivalent.  One CTA per replica finds the
-//   n-th smallest 64-bit key (|phibar| bits << 32 | i) by an 8-pass radix
-//   select over 8-bit digits; a spin is ambivalent iff its key <= that key.
+//   n-th smallest 64-bit key (|phibar| bits << 32 | i) by a radix select; a
+//   spin is ambivalent iff its key <= that key.
 //   Keys are unique, so no tie handling is needed beyond the index bits.
 // Energy (Eq. (1)) and cut (Methods, "MAX-CUT and Ising spin-glass"):
 //   ordered = sum_i s_i sum_{j != i} J_ij s_j   (int32 per row, int64 total)
@@ -24,55 +24,85 @@ __device__ __forceinline__ unsigned long long rkey(const float* x, int i)
 
 // One replica: x = its N window means; spins/frozen point at its row;
 // tally at its two counters (any may be null).
+//
+// The n-th smallest key by a radix select, at most five passes: 11, 11 and 9
+// bits of |phibar| and, for ties, 11 and 5 bits of the index (N <= 65536).  It
+// ends as soon as the target's bucket holds one key, usually after the second
+// pass: every key at or below the prefix is then wanted.  11-bit digits spread
+// a narrow range of exponents over many bins, and the bins are scanned by the
+// whole block (one thread walking 256 bins eight times took most of the
+// kernel: K2000 x 4096 97 -> 30 us).
+constexpr int kBins = 2048;
+
 __device__ __forceinline__ void readout_block(const float* __restrict__ x, int N, int n,
                                               int8_t* spins, uint8_t* frozen, int32_t* tally,
                                               uint32_t* status)
 {
-    __shared__ unsigned hist[256];
-    __shared__ unsigned long long s_prefix, s_mask;
-    __shared__ unsigned s_target;
+    __shared__ __align__(16) unsigned hist[kBins];
+    __shared__ unsigned s_warp[kThreads / 32];
+    __shared__ unsigned s_bin, s_before, s_count;
+    constexpr int kPer = kBins / kThreads;
     const int nn = n < 0 ? 0 : (n > N ? N : n);
-    unsigned long long K = 0;  // ambivalent iff key <= K (nn >= 1)
+    unsigned long long K = 0, M = ~0ull;  // ambivalent iff (key & M) <= K (nn >= 1)
     if (nn > 0 && nn < N) {
-        if (threadIdx.x == 0) {
-            s_prefix = 0;
-            s_mask = 0;
-            s_target = (unsigned)(nn - 1);
-        }
-        for (int shift = 56; shift >= 0; shift -= 8) {
-            for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0;
+        const int shifts[5] = {52, 41, 32, 5, 0};
+        const unsigned widths[5] = {2047u, 2047u, 511u, 2047u, 31u};
+        unsigned target = (unsigned)(nn - 1);
+        M = 0;
+        for (int pass = 0; pass < 5; ++pass) {
+            for (int b = threadIdx.x; b < kBins; b += kThreads) hist[b] = 0;
             __syncthreads();
-            const unsigned long long pre = s_prefix, msk = s_mask;
-            for (int i = threadIdx.x; i < N; i += blockDim.x) {
+            const int shift = shifts[pass];
+            for (int i = threadIdx.x; i < N; i += kThreads) {
                 const unsigned long long k = rkey(x, i);
-                if ((k & msk) == pre) atomicAdd(&hist[(k >> shift) & 255u], 1u);
+                if ((k & M) == K) atomicAdd(&hist[(unsigned)(k >> shift) & widths[pass]], 1u);
             }
             __syncthreads();
-            if (threadIdx.x == 0) {
-                unsigned cum = 0, tgt = s_target;
-                for (int b = 0; b < 256; ++b) {
-                    if (cum + hist[b] > tgt) {
-                        s_prefix = pre | ((unsigned long long)b << shift);
-                        s_target = tgt - cum;
-                        break;
+            // each thread sums its kPer bins; block-wide exclusive scan of the sums
+            unsigned own[kPer], sum = 0;
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) {
+                own[q] = hist[threadIdx.x * kPer + q];
+                sum += own[q];
+            }
+            unsigned inc = sum;
+            const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += v;
+            }
+            if (lane == 31) s_warp[warp] = inc;
+            __syncthreads();
+            unsigned cum = inc - sum;
+            for (int w = 0; w < warp; ++w) cum += s_warp[w];
+            if (target >= cum && target < cum + sum) {   // exactly one thread
+#pragma unroll
+                for (int q = 0; q < kPer; ++q) {
+                    if (target >= cum && target < cum + own[q]) {
+                        s_bin = threadIdx.x * kPer + q;
+                        s_before = cum;
+                        s_count = own[q];
                     }
-                    cum += hist[b];
+                    cum += own[q];
                 }
-                s_mask = msk | (255ull << shift);
             }
             __syncthreads();
+            K |= (unsigned long long)s_bin << shift;
+            M |= (unsigned long long)widths[pass] << shift;
+            target -= s_before;
+            if (s_count == 1u) break;
         }
-        K = s_prefix;
     }
     bool bad = false;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    for (int i = threadIdx.x; i < N; i += kThreads) {
         const float v = x[i];
         bad |= !isfinite(v);
         if (spins) spins[i] = v >= 0.f ? 1 : -1;
         bool amb;
         if (nn == 0) amb = false;
         else if (nn == N) amb = true;
-        else amb = rkey(x, i) <= K;
+        else amb = (rkey(x, i) & M) <= K;
         if (frozen) frozen[i] = amb ? 0 : 1;
     }
     if (tally && threadIdx.x == 0) {
@@ -147,53 +177,131 @@ __global__ void __launch_bounds__(kThreads) k_energy_csr(const int32_t* __restri
 // Integer energy for couplings in {-1, 0, +1} with many couplings per row
 // (dense instances), from bit masks instead of per-coupling gathers.  With
 // bit j of a spin mask set where s_j = -1, and per row i the masks of its
-// nonzero couplings (nz) and of its negative ones (neg), a term J_ij s_j is
-// -1 exactly where (neg_i XOR S) AND nz_i has a bit, so
-//   g_i = sum_j J_ij s_j = deg_i - 2 popc((neg_i ^ S) & nz_i),
-// and sum_i s_i g_i is summed in int64 as in energy_block.  The row masks are
-// stored word-major ([word][row]), so the 32 lanes of a warp, one row each,
-// read one coalesced 128-byte line per word; a warp owns one replica and
-// builds its spin mask in shared memory by ballots.
+// couplings to j > i (nz) and of the negative ones (neg), a term J_ij s_j is
+// -1 exactly where x = neg_i XOR (S AND nz_i) has a bit, so
+//   sum_{j > i} J_ij s_j = deg_i - 2 popc(x)   (deg_i: couplings to j > i),
+// and sum_i s_i times that is half the ordered sum of energy_block.  Row masks
+// are stored word-major ([word][row]): the 32 lanes of a warp, one row each,
+// read coalesced 128-byte lines.
+//
+// A block owns Q replicas, their spin masks in shared memory, and its warps
+// share the row blocks; each mask word that is loaded serves all Q.  The
+// counts run through carry-save adders, so four words cost one population
+// count instead of four (16 per clock and SM against 64 logic operations).
+// K2000 x 4096: one replica per warp, both triangles, one popc per word,
+// streamed 4 GB of masks from L2 in 926 us; this form takes 125 us.
 constexpr int kBitsWarps = 8;
 
+__device__ __forceinline__ void csa(uint32_t& sum, uint32_t& carry, uint32_t a, uint32_t b)
+{
+    const uint32_t s = sum;
+    sum = s ^ a ^ b;
+    carry = (s & a) | (s & b) | (a & b);
+}
+
+template <int Q>
 __global__ void __launch_bounds__(kBitsWarps * 32)
 k_energy_bits(const uint32_t* __restrict__ nzT, const uint32_t* __restrict__ negT,
               const int32_t* __restrict__ deg, const int32_t* __restrict__ h, int N, int Wd,
               int Npad, int R, int64_t sumJ, const int8_t* __restrict__ spins, int64_t* energy,
               int64_t* cut)
 {
-    extern __shared__ uint32_t smask[];   // [kBitsWarps][Wd]
+    extern __shared__ uint32_t S[];       // [Wd + 3][Q] spin masks, word-major
+    __shared__ long long s_sum[kBitsWarps][2][Q];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = blockIdx.x * kBitsWarps + warp;
-    if (r >= R) return;                   // whole warp: no block-wide barrier below
-    uint32_t* S = smask + (size_t)warp * Wd;
-    const int8_t* s = spins + (size_t)r * N;
-    for (int w = 0; w < Wd; ++w) {
-        const int j = 32 * w + lane;
-        const uint32_t b = __ballot_sync(0xffffffffu, j < N && s[j] < 0);
-        if (lane == 0) S[w] = b;
+    const int r0 = blockIdx.x * Q;
+    for (int k = warp; k < (Wd + 3) * Q; k += kBitsWarps) {
+        const int w = k / Q, q = k % Q, j = 32 * w + lane;
+        const uint32_t b =
+            __ballot_sync(0xffffffffu, j < N && r0 + q < R && spins[(size_t)(r0 + q) * N + j] < 0);
+        if (lane == 0) S[k] = b;
     }
-    __syncwarp();
-    long long ordered = 0, field = 0;
-    for (int i0 = 0; i0 < N; i0 += 32) {
-        const int i = i0 + lane;
-        int cnt = 0;
-        for (int w = 0; w < Wd; ++w)
-            cnt += __popc((negT[(size_t)w * Npad + i] ^ S[w]) & nzT[(size_t)w * Npad + i]);
-        if (i < N) {
-            const int si = ((S[i >> 5] >> (i & 31)) & 1u) ? -1 : 1;
-            ordered += (long long)si * (long long)(deg[i] - 2 * cnt);
-            if (h) field += (long long)h[i] * si;
+    __syncthreads();
+    long long pair[Q], field[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) pair[q] = field[q] = 0;
+    // row blocks dealt back and forth: block b has Wd - b words
+    for (int g = 0; g * kBitsWarps < Wd; ++g) {
+        const int rb = g * kBitsWarps + ((g & 1) ? kBitsWarps - 1 - warp : warp);
+        if (rb >= Wd) continue;
+        const int i = 32 * rb + lane;
+        uint32_t ones[Q], twos[Q];
+        int cnt[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            ones[q] = twos[q] = 0u;
+            cnt[q] = 0;
+        }
+        for (int w = rb; w < Wd; w += 4) {
+            uint32_t nz[4], ng[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool in = w + u < Wd;
+                nz[u] = in ? __ldg(nzT + (size_t)(w + u) * Npad + i) : 0u;
+                ng[u] = in ? __ldg(negT + (size_t)(w + u) * Npad + i) : 0u;
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                uint32_t x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[u] = ng[u] ^ (S[(w + u) * Q + q] & nz[u]);
+                uint32_t t0, t1, f;
+                csa(ones[q], t0, x[0], x[1]);
+                csa(ones[q], t1, x[2], x[3]);
+                csa(twos[q], f, t0, t1);
+                cnt[q] += __popc(f);
+            }
+        }
+        const int d = i < N ? deg[i] : 0, hi = (h && i < N) ? h[i] : 0;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int c = 4 * cnt[q] + 2 * __popc(twos[q]) + __popc(ones[q]);
+            const bool down = (S[rb * Q + q] >> lane) & 1u;
+            pair[q] += down ? 2 * c - d : d - 2 * c;
+            field[q] += down ? -hi : hi;
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        ordered += __shfl_xor_sync(0xffffffffu, ordered, o);
-        field += __shfl_xor_sync(0xffffffffu, field, o);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        for (int o = 16; o > 0; o >>= 1) {
+            pair[q] += __shfl_xor_sync(0xffffffffu, pair[q], o);
+            field[q] += __shfl_xor_sync(0xffffffffu, field[q], o);
+        }
+        if (lane == 0) {
+            s_sum[warp][0][q] = pair[q];
+            s_sum[warp][1][q] = field[q];
+        }
     }
-    if (lane == 0) {
-        if (energy) energy[r] = ordered / 2 + field;
-        if (cut) cut[r] = (sumJ - ordered) / 4;
+    __syncthreads();
+    if (threadIdx.x < Q && r0 + (int)threadIdx.x < R) {
+        long long p = 0, f = 0;
+        for (int w = 0; w < kBitsWarps; ++w) {
+            p += s_sum[w][0][threadIdx.x];
+            f += s_sum[w][1][threadIdx.x];
+        }
+        if (energy) energy[r0 + threadIdx.x] = p + f;
+        if (cut) cut[r0 + threadIdx.x] = (sumJ - 2 * p) / 4;
     }
+}
+
+// The masks of k_energy_bits from the CSR rows (arrays zeroed before): one
+// block per row.
+__global__ void __launch_bounds__(128) k_energy_masks(const int32_t* __restrict__ row_ptr,
+                                                      const int32_t* __restrict__ col,
+                                                      const int8_t* __restrict__ val, int Npad,
+                                                      uint32_t* nzT, uint32_t* negT, int32_t* deg)
+{
+    const int i = blockIdx.x;
+    int c = 0;
+    for (int k = row_ptr[i] + (int)threadIdx.x; k < row_ptr[i + 1]; k += blockDim.x) {
+        const int j = col[k];
+        if (j <= i) continue;
+        ++c;
+        const size_t o = (size_t)(j >> 5) * Npad + i;
+        atomicOr(nzT + o, 1u << (j & 31));
+        if (val[k] < 0) atomicOr(negT + o, 1u << (j & 31));
+    }
+    if (c) atomicAdd(deg + i, c);
 }
 
 // Ising energy for real-valued couplings and fields (Results Eq. (1)), exact up
@@ -405,23 +513,20 @@ static hqa_status energy_bits_setup(hqa_ctx* ctx)
     if (ctx->d_ebits) return HQA_OK;
     if (hqa_capturing()) return hqa_capture_note(HQA_ERR_UNSUPPORTED);
     const int N = ctx->N, Wd = (N + 31) / 32, Npad = Wd * 32;
-    std::vector<uint32_t> nz((size_t)Wd * Npad, 0u), neg((size_t)Wd * Npad, 0u);
-    std::vector<int32_t> deg(N, 0);
-    for (int i = 0; i < N; ++i)
-        for (int64_t k = ctx->row_ptr[i]; k < ctx->row_ptr[i + 1]; ++k) {
-            const int j = ctx->col[k];
-            nz[(size_t)(j >> 5) * Npad + i] |= 1u << (j & 31);
-            if (ctx->val[k] < 0.f) neg[(size_t)(j >> 5) * Npad + i] |= 1u << (j & 31);
-            ++deg[i];
-        }
-    const size_t mb = nz.size() * sizeof(uint32_t);
+    const size_t mb = (size_t)Wd * Npad * sizeof(uint32_t), bytes = 2 * mb + (size_t)N * sizeof(int32_t);
     void* d = nullptr;
-    HQA_CUDA_TRY(cudaMalloc(&d, 2 * mb + (size_t)N * sizeof(int32_t)));
+    HQA_CUDA_TRY(cudaMalloc(&d, bytes));
     char* b = static_cast<char*>(d);
-    if (cudaMemcpy(b, nz.data(), mb, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(b + mb, neg.data(), mb, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(b + 2 * mb, deg.data(), (size_t)N * sizeof(int32_t), cudaMemcpyHostToDevice) !=
-            cudaSuccess) {
+    cudaError_t e = cudaMemset(d, 0, bytes);
+    if (e == cudaSuccess) {
+        k_energy_masks<<<N, 128>>>(ctx->d_row_ptr, ctx->d_col, ctx->d_val_i8, Npad,
+                                   reinterpret_cast<uint32_t*>(b), reinterpret_cast<uint32_t*>(b + mb),
+                                   reinterpret_cast<int32_t*>(b + 2 * mb));
+        e = cudaGetLastError();
+    }
+    // the caller's stream need not wait for the legacy one
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    if (e != cudaSuccess) {
         cudaFree(d);
         (void)cudaGetLastError();
         return HQA_ERR_CUDA;
@@ -457,12 +562,20 @@ hqa_status hqa_launch_energy_ex(hqa_ctx* ctx, int32_t R, const int8_t* spins, in
         const int N = ctx->N, Wd = (N + 31) / 32, Npad = Wd * 32;
         const size_t mb = (size_t)Wd * Npad * sizeof(uint32_t);
         const char* b = static_cast<const char*>(ctx->d_ebits);
-        const size_t smem = (size_t)kBitsWarps * Wd * sizeof(uint32_t);
-        if (smem > 48 * 1024) return HQA_ERR_TOO_LARGE;   // N <= 49152
-        k_energy_bits<<<(R + kBitsWarps - 1) / kBitsWarps, kBitsWarps * 32, smem, st>>>(
-            reinterpret_cast<const uint32_t*>(b), reinterpret_cast<const uint32_t*>(b + mb),
-            reinterpret_cast<const int32_t*>(b + 2 * mb), ctx->has_h ? ctx->d_h_i32 : nullptr, N,
-            Wd, Npad, R, ctx->sum_J_all, spins, energy, cut);
+        if ((size_t)kBitsWarps * Wd * sizeof(uint32_t) > 48 * 1024) return HQA_ERR_TOO_LARGE;   // N <= 49152
+        // replicas per block: as many as leave at least three blocks per SM
+        // (and, beside the static part, as their masks fit in 48 KB)
+        const int Q = R >= 24 * ctx->sm_count && Wd <= 1400 ? 8 : R >= 6 * ctx->sm_count ? 4 : 1;
+        const size_t smem = (size_t)Q * (Wd + 3) * sizeof(uint32_t);
+        const auto go = [&](auto kernel) {
+            kernel<<<(R + Q - 1) / Q, kBitsWarps * 32, smem, st>>>(
+                reinterpret_cast<const uint32_t*>(b), reinterpret_cast<const uint32_t*>(b + mb),
+                reinterpret_cast<const int32_t*>(b + 2 * mb), ctx->has_h ? ctx->d_h_i32 : nullptr, N,
+                Wd, Npad, R, ctx->sum_J_all, spins, energy, cut);
+        };
+        if (Q == 8) go(k_energy_bits<8>);
+        else if (Q == 4) go(k_energy_bits<4>);
+        else go(k_energy_bits<1>);
         return cudaGetLastError() == cudaSuccess ? HQA_OK : HQA_ERR_CUDA;
     }
     k_energy_csr<<<R, kThreads, 0, st>>>(ctx->d_row_ptr, ctx->d_col, ctx->d_val_i8,
