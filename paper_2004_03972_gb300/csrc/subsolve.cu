@@ -23,6 +23,11 @@
 // re-walks only the threads that reached the replica minimum and keeps the
 // smallest x attaining it.  Replicas outside the 16-bit bound, or with
 // fewer than 3 walked bits, take the scalar walk.
+//
+// Before either walk k_sub_reduce shrinks the problem without losing the
+// optimum.  The ambivalent spins of a sparse graph hold few couplings among
+// themselves, so most of them are decided by their field or hang off one
+// neighbour, and the rest falls into small components.
 #include <algorithm>
 #include <atomic>
 #include <mutex>
@@ -37,7 +42,7 @@ constexpr int kEnumThreads = 256;
 
 struct SubPrep {
     int32_t n;          // ambivalent count, -1 if invalid
-    int32_t packed;     // 1: the packed 16-bit walk solves this replica
+    int32_t packed;     // 0: scalar walk, 1: packed 16-bit walk, 2: solved by k_sub_reduce
     int32_t amb[32];    // spin index of a_k
     int32_t heff[32];
     uint32_t nz[32];
@@ -379,7 +384,7 @@ __device__ __forceinline__ bool load_packed(const SubPrep* P, uint32_t* s_nz, ui
                                             uint32_t* s_nA, uint32_t* s_nB)
 {
     const int n = P->n;
-    if (n < 0 || !P->packed) return false;
+    if (n < 0 || P->packed != 1) return false;
     for (int a = threadIdx.x; a < 32; a += blockDim.x) {
         const bool v = a < n;
         const uint32_t nz = v ? P->nz[a] : 0u, ng = v ? P->neg[a] : 0u;
@@ -462,6 +467,183 @@ __global__ void __launch_bounds__(kEnumThreads) k_sub_enum16_arg(const SubPrep* 
     }
 }
 
+// Exact reduction, one CTA per replica.  The problem is minimised with its tie
+// break built in: E(s) = 2^33 H'(s) - sum_k 2^k s_k has one minimum, the
+// optimum with the smallest x (2^33 exceeds what the second sum can change), so
+// every rule below may decide spins in any order.  Lane k of warp 0 holds spin
+// k's field and coupling masks; until nothing changes,
+//   - a spin whose |field| exceeds the sum of its open |couplings| takes the
+//     sign against its field, whatever the others do (|h| > deg);
+//   - a spin with one open neighbour j is minimised out: -|h + J s_j| is linear
+//     in s_j and goes into j's field; its sign follows from s_j afterwards.
+// What is left splits into connected components, each enumerated by the CTA in
+// Gray order, 2^(c - 8) steps per thread.  A component of more than 12 spins is
+// solved here only when it is at least 4 spins smaller than the whole problem:
+// a step here takes about ten times the packed walk's 1.2 instructions per
+// configuration, so up to there this is the shorter way; the walks get the rest
+// (complete graphs).  ER800 x 1024, n = 24 (16.8 M configurations, of which the
+// reduction leaves a few hundred): 3.1 ms of walks before, 21 us.
+constexpr int kTieShift = 33;
+
+__global__ void __launch_bounds__(kEnumThreads) k_sub_reduce(SubPrep* __restrict__ prep,
+                                                             unsigned long long* keys)
+{
+    __shared__ long long s_h[32], s_red[kEnumThreads / 32];
+    __shared__ uint32_t s_nz[32], s_ng[32], s_comp[32], s_redx[kEnumThreads / 32], s_S;
+    __shared__ int s_ncomp, s_solve;
+    SubPrep* P = prep + blockIdx.x;
+    const int n = P->n;
+    if (n < 0) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long h = 0, out_h = 0;                    // warp 0: lane k's spin
+    uint32_t nz = 0, ng = 0, core = 0, S = 0;      // S bit k: s_k = -1
+    int iters = 0, out_iter = -1, out_nb = 0;      // when and onto whom it was minimised out
+    const long long J = 1ll << kTieShift;
+    if (warp == 0) {
+        if (lane < n) {
+            nz = P->nz[lane];
+            ng = P->neg[lane];
+            h = (long long)P->heff[lane] * J - (1ll << lane);
+        }
+        core = (1u << n) - 1u;                     // n <= 30
+        for (;; ++iters) {
+            bool on = (core >> lane) & 1u;
+            const bool fix = on && llabs(h) > (long long)__popc(nz & core) * J;
+            const uint32_t F = __ballot_sync(0xffffffffu, fix);
+            S |= __ballot_sync(0xffffffffu, fix && h > 0);
+            core &= ~F;
+            const uint32_t mF = nz & F;
+            h += (long long)(__popc(mF) - 2 * __popc((ng ^ S) & mF)) * J;
+            on = (core >> lane) & 1u;
+            const uint32_t open = nz & core;
+            const bool leaf = on && __popc(open) == 1;
+            const uint32_t L = __ballot_sync(0xffffffffu, leaf);
+            const int nb = leaf ? __ffs(open) - 1 : 0;
+            const bool out = leaf && !(((L >> nb) & 1u) && nb < lane);   // of a lone pair, the lower
+            const uint32_t E = __ballot_sync(0xffffffffu, out);
+            if (!(F | E)) break;
+            const long long Jl = ((ng >> nb) & 1u) ? -J : J;
+            const long long b = (llabs(h + Jl) - llabs(h - Jl)) / 2;
+            for (uint32_t e = E; e; e &= e - 1) {
+                const int src = __ffs(e) - 1;
+                const long long bs = __shfl_sync(0xffffffffu, b, src);
+                if (lane == __shfl_sync(0xffffffffu, nb, src)) h -= bs;
+            }
+            if (out) {
+                out_iter = iters;
+                out_nb = nb;
+                out_h = h;
+            }
+            core &= ~E;
+        }
+        // connected components of what is left
+        int nc = 0, most = 0;
+        for (uint32_t rest = core; rest; ++nc) {
+            uint32_t c = rest & (0u - rest), c0;
+            do {
+                c0 = c;
+                c |= __reduce_or_sync(0xffffffffu, ((c >> lane) & 1u) ? (nz & core) : 0u);
+            } while (c != c0);
+            if (lane == 0) s_comp[nc] = c;
+            most = max(most, __popc(c));
+            rest &= ~c;
+        }
+        if (lane == 0) {
+            s_ncomp = nc;
+            s_solve = most <= 12 || most <= n - 4;
+            s_S = 0;
+        }
+    }
+    __syncthreads();
+    if (!s_solve) return;
+    const int ncomp = s_ncomp;
+    for (int q = 0; q < ncomp; ++q) {
+        const uint32_t C = s_comp[q];
+        const int c = __popc(C);
+        if (warp == 0 && ((C >> lane) & 1u)) {
+            // compact the component's spins to 0 .. c - 1
+            const int a = __popc(C & ((1u << lane) - 1u));
+            uint32_t z = 0, g = 0;
+            int b = 0;
+            for (uint32_t m = C; m; m &= m - 1, ++b) {
+                const int j = __ffs(m) - 1;
+                z |= ((nz >> j) & 1u) << b;
+                g |= ((ng >> j) & 1u) << b;
+            }
+            s_h[a] = h;
+            s_nz[a] = z;
+            s_ng[a] = g;
+        }
+        __syncthreads();
+        const int LB = c > 8 ? c - 8 : 0;
+        long long best = 0x7fffffffffffffffll;
+        uint32_t bx = 0;
+        if (threadIdx.x < (1u << (c - LB))) {
+            uint32_t x = threadIdx.x << LB;
+            long long pair2 = 0, E = 0;
+            for (int a = 0; a < c; ++a) {
+                const int g = __popc(s_nz[a]) - 2 * __popc((s_ng[a] ^ x) & s_nz[a]);
+                const bool down = (x >> a) & 1u;
+                pair2 += down ? -g : g;
+                E += down ? -s_h[a] : s_h[a];
+            }
+            E += pair2 / 2 * J;
+            best = E;
+            bx = x;
+            for (uint32_t t = 1; t < (1u << LB); ++t) {
+                const int k = __ffs(t) - 1;
+                const uint32_t z = s_nz[k];
+                const int g = __popc(z) - 2 * __popc((s_ng[k] ^ x) & z);
+                const long long d = 2 * ((long long)g * J + s_h[k]);
+                E += ((x >> k) & 1u) ? d : -d;
+                x ^= 1u << k;
+                if (E < best) {
+                    best = E;
+                    bx = x;
+                }
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long e2 = __shfl_xor_sync(0xffffffffu, best, o);
+            const uint32_t x2 = __shfl_xor_sync(0xffffffffu, bx, o);
+            if (e2 < best) {
+                best = e2;
+                bx = x2;
+            }
+        }
+        if (lane == 0) {
+            s_red[warp] = best;
+            s_redx[warp] = bx;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < kEnumThreads / 32; ++w)
+                if (s_red[w] < best) {
+                    best = s_red[w];
+                    bx = s_redx[w];
+                }
+            uint32_t m = C;
+            for (int a = 0; a < c; ++a, m &= m - 1)
+                if ((bx >> a) & 1u) s_S |= m & (0u - m);
+        }
+        __syncthreads();
+    }
+    if (warp == 0) {
+        S |= s_S;
+        // the spins minimised out, last ones first
+        for (int it = iters - 1; it >= 0; --it) {
+            const long long Jl = ((ng >> out_nb) & 1u) ? -J : J;
+            const bool mine = out_iter == it;
+            const bool down = mine && out_h + (((S >> out_nb) & 1u) ? -Jl : Jl) > 0;
+            S |= __ballot_sync(0xffffffffu, down);
+        }
+        if (lane == 0) {
+            keys[blockIdx.x] = S;
+            P->packed = 2;
+        }
+    }
+}
+
 // Writes the assembled configuration.
 __global__ void k_sub_assemble(const SubPrep* __restrict__ prep,
                                const unsigned long long* __restrict__ keys, int N,
@@ -518,6 +700,7 @@ hqa_status hqa_launch_subsolve(hqa_ctx* ctx, int32_t R, const int8_t* spins,
     k_sub_prep<<<R, kPrepThreads, 0, st>>>(ctx->d_row_ptr, ctx->d_col, ctx->d_val_i8,
                                            ctx->has_h ? ctx->d_h_i32 : nullptr, ctx->N, n, spins,
                                            frozen, prep, keys, ctx->d_status, 1, emin);
+    k_sub_reduce<<<R, kEnumThreads, 0, st>>>(prep, keys);
     k_sub_enum16_min<<<grid, kEnumThreads, 0, st>>>(prep, LB, tmin, emin);
     k_sub_enum16_arg<<<grid, kEnumThreads, 0, st>>>(prep, LB, tmin, emin, keys);
     k_sub_enum<<<grid, kEnumThreads, 0, st>>>(prep, LB, keys);
