@@ -314,6 +314,8 @@ def kernel_name(hqa, plan, prec_name):
         if prec_name == "PREC_FP32":
             # 256 threads: the CUDA-core form; else the fixed-point slices on the tensor cores
             return "k_dense_simt<1>" if plan.get("threads", 256) == 256 else "k_dense_f32"
+        if plan.get("threads") == 320:
+            return "k_dense_wide"
         kseg = 2 if prec_name.endswith("X2") else 1
         f16 = "true" if prec_name.startswith("PREC_FP16") else "false"
         return f"k_dense_md<{plan['replicas_per_block'] // 2},*,{kseg},*,*,{f16},*,*,*>"

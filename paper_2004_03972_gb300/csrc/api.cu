@@ -886,6 +886,19 @@ hqa_status hqa_plan_query(hqa_ctx* ctx, int32_t replicas, const hqa_run_opts* op
         int nh = 0, grid = 0;
         const int C = hqa_dense_md_chunks(ctx, replicas, o.precision);
         const int Rc = (replicas + C - 1) / C;
+        if (hqa_dense_wide(ctx, replicas, o.precision)) {
+            const int units = (ctx->N + 255) / 256 * ((Rc + 255) / 256);
+            out->kernel = HQA_KERNEL_DENSE;
+            out->replicas_per_block = 256;
+            out->blocks = 2 * std::min(units, ctx->sm_count / 2);
+            out->threads = 320;     // TMA warp, MMA warp, 8 epilogue warps
+            out->smem_bytes = 0;
+            out->chunks = C;
+            out->pad_ratio = (double)C * units * 256 * 256 / ((double)ctx->N * replicas);
+            out->conflict_ratio = 1.0;
+            out->balance = 1.0;
+            return HQA_OK;
+        }
         if (!hqa_dense_md_geometry(ctx, Rc, &nh, &grid)) return HQA_ERR_UNSUPPORTED;
         out->kernel = HQA_KERNEL_DENSE;
         out->replicas_per_block = 2 * nh;

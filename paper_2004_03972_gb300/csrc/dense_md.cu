@@ -440,16 +440,33 @@ int hqa_dense_md_geometry(const hqa_ctx* ctx, int32_t R, int* nh, int* grid)
     return 1;
 }
 
-static hqa_status dense_md_chunk(hqa_ctx* ctx, const StepCoef* d_sched, int64_t S, int32_t W,
+constexpr int kWideMost = 8192;   // replicas per launch: bounds its state (24 bytes or more each and spin)
+
+// Whether a run takes the 256 x 256 units of dense_wide.cu: where one CTA per row
+// tile leaves column tiles too wide for their state on chip, or, with so many row
+// tiles that at most three column groups fit (N > 4864), needs several runs one
+// after another.  us per step, one CTA per row tile / units: N = 10000 x 1024
+// BF16x2 714 / 486, 7000 x 2048 FP16x2 431 / 228, 6000 x 1000 BF16 75 / 55, 5000 x
+// 1000 FP16x2 128 / 72.  Below, the state on chip and the shorter chain of a step
+// win: 7000 x 520 FP16x2 95.5 / 98, 5000 x 400 BF16 34 / 42, 2000 x 4096 FP16x2 45 / 49.
+bool hqa_dense_wide(const hqa_ctx* ctx, int32_t R, int prec)
+{
+    const int C = dense_chunks(ctx, R, prec);
+    int NH = 0, grid = 0;
+    if (!hqa_dense_md_geometry(ctx, (R + C - 1) / C, &NH, &grid)) return false;
+    return NH > 160 || (C > 1 && ctx->Mpad / BM > 38);
+}
+
+static hqa_status dense_md_chunk(hqa_ctx* ctx, bool wide, const StepCoef* d_sched, int64_t S, int32_t W,
                                  int32_t R, int32_t rep0, uint64_t seed, int init,
                                  const float* phi0, const float* p0, int M, float* phi_out,
                                  float* p_out, float* phibar_out, int prec, cudaStream_t st)
 {
-    int NH = 0, grid = 0;
-    if (!hqa_dense_md_geometry(ctx, R, &NH, &grid)) return HQA_ERR_TOO_LARGE;
+    int NH = hqa_wide_block() / 2, grid = 0;
+    if (!wide && !hqa_dense_md_geometry(ctx, R, &NH, &grid)) return HQA_ERR_TOO_LARGE;
     const bool f16 = is_f16(prec);
     const int Mt = ctx->Mpad / BM;
-    const int Nc = grid / Mt;
+    const int Nc = wide ? (R + 2 * NH - 1) / (2 * NH) : grid / Mt;   // column groups or blocks
     const int Rpad = Nc * 2 * NH;
     const int Npad = ctx->Mpad;
     const size_t n = (size_t)Rpad * Npad;
@@ -490,7 +507,7 @@ static hqa_status dense_md_chunk(hqa_ctx* ctx, const StepCoef* d_sched, int64_t 
     }
     CUtensorMap tmB;
     // a CTA of a pair stages half of each NH-replica phi tile
-    const uint32_t box_rows = hqa_dense::use_pair(NH, Mt) ? NH / 2 : NH;
+    const uint32_t box_rows = wide ? hqa_wide_block() / 2 : hqa_dense::use_pair(NH, Mt) ? NH / 2 : NH;
     if (!make_tmap16(&tmB, a.phib, (uint64_t)2 * Rpad, (uint64_t)kseg * Npad, box_rows, f16))
         return HQA_ERR_CUDA;
     // the epilogue's operand stores: 128 spins x 16 replicas per box, unswizzled
@@ -504,7 +521,8 @@ static hqa_status dense_md_chunk(hqa_ctx* ctx, const StepCoef* d_sched, int64_t 
     else hqa_dense::k_dense_init<false><<<g, 256, 0, st>>>(a, seed, init, phi0, p0, kseg);
     if (cudaMemsetAsync(a.gbar, 0, (size_t)2 * Nc * sizeof(unsigned int), st) != cudaSuccess)
         return HQA_ERR_CUDA;
-    s = f16 ? hqa_dense::dense_md_dispatch<true>(ctx, a, NH, kseg, grid, st, tmA, tmB, tmS)
+    s = wide ? hqa_wide_launch(ctx, a, kseg, f16, st, tmA, tmB)
+      : f16 ? hqa_dense::dense_md_dispatch<true>(ctx, a, NH, kseg, grid, st, tmA, tmB, tmS)
             : hqa_dense::dense_md_dispatch<false>(ctx, a, NH, kseg, grid, st, tmA, tmB, tmS);
     if (s != HQA_OK) return s;
     const int64_t nwin = S < W ? S : W;
@@ -515,6 +533,7 @@ static hqa_status dense_md_chunk(hqa_ctx* ctx, const StepCoef* d_sched, int64_t 
 
 int hqa_dense_md_chunks(const hqa_ctx* ctx, int32_t R, int prec)
 {
+    if (hqa_dense_wide(ctx, R, prec)) return (R + kWideMost - 1) / kWideMost;
     return dense_chunks(ctx, R, prec);
 }
 
@@ -525,13 +544,14 @@ hqa_status hqa_dense_launch_md(hqa_ctx* ctx, const StepCoef* d_sched, int64_t S,
 {
     hqa_status s = hqa_dense_prepare(ctx, prec);
     if (s != HQA_OK) return s;
-    const int C = dense_chunks(ctx, R, prec);
+    const bool wide = hqa_dense_wide(ctx, R, prec);
+    const int C = hqa_dense_md_chunks(ctx, R, prec);
     const int Rc = (R + C - 1) / C;
     const size_t N = (size_t)ctx->N;
     for (int r0 = 0; r0 < R; r0 += Rc) {
         const int Rk = std::min(Rc, R - r0);
         const size_t o = (size_t)r0 * N;
-        s = dense_md_chunk(ctx, d_sched, S, W, Rk, r0, seed, init, phi0 ? phi0 + o : nullptr,
+        s = dense_md_chunk(ctx, wide, d_sched, S, W, Rk, r0, seed, init, phi0 ? phi0 + o : nullptr,
                            p0 ? p0 + o : nullptr, M, phi_out ? phi_out + o : nullptr,
                            p_out ? p_out + o : nullptr, phibar_out ? phibar_out + o : nullptr,
                            prec, st);

@@ -152,6 +152,15 @@ struct DenseMDArgs {
     uint64_t wait_ns;
 };
 
+}  // namespace hqa_dense
+
+// dense_wide.cu: 256 x 256 units dealt to CTA pairs (large instances)
+int hqa_wide_block();
+hqa_status hqa_wide_launch(hqa_ctx* ctx, const hqa_dense::DenseMDArgs& a, int kseg, bool f16,
+                           cudaStream_t st, const CUtensorMap& tmA, const CUtensorMap& tmB);
+
+namespace hqa_dense {
+
 static __device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p)
 {
     unsigned int v;

@@ -295,6 +295,7 @@ hqa_status hqa_dense_field(hqa_ctx* ctx, int32_t R, const float* phi, float* L, 
                            cudaStream_t st);
 bool hqa_dense_md_possible(const hqa_ctx* ctx, int32_t R);
 int hqa_dense_md_geometry(const hqa_ctx* ctx, int32_t R, int* nh, int* grid);
+bool hqa_dense_wide(const hqa_ctx* ctx, int32_t R, int prec);
 int hqa_dense_md_chunks(const hqa_ctx* ctx, int32_t R, int prec);
 // precision: HQA_PREC_BF16, _BF16X2, _FP16 or _FP16X2
 bool hqa_tc_precision(int prec);
