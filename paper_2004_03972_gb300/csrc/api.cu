@@ -448,7 +448,8 @@ hqa_status run_batch(hqa_ctx* ctx, const hqa_schedule* sched, double dt, int64_t
     const float* p0 = o.init == HQA_INIT_GIVEN ? o.p0 : nullptr;
     if (kern == HQA_KERNEL_LOWDEG)
         s = hqa_lowdeg_launch_md(ctx, RB, o.precision, ctx->d_sched, steps, sched->window, replicas,
-                                 seed, o.init, phi0, p0, sched->M, out->phi, out->p, phibar, st);
+                                 seed, o.init, phi0, p0, sched->M, out->phi, out->p, phibar,
+                                 o.replicas_per_block == 0, st);
     else
         s = hqa_batch_launch_md(ctx, RB, o.precision, ctx->d_sched, steps, sched->window, replicas,
                                 seed, o.init, phi0, p0, sched->M, out->phi, out->p, phibar, st);

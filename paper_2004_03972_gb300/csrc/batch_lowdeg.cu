@@ -39,6 +39,31 @@ __host__ __device__ constexpr uint32_t ld_item_bytes(int N, int RB, bool bf16, b
            align16((uint32_t)N * 8u) + (has_h ? align16((uint32_t)N * 4u) : 0u);
 }
 
+// Register-resident form: units (a spin and 2 replicas at RB = 2, 4 above) per
+// thread that its registers hold without spilling, and the shared memory of its
+// operand (two step buffers, each row and its negative).
+__host__ __device__ constexpr int ld_reg_units(int N, int RB)
+{
+    return (N * (RB >= 8 ? RB / 4 : 1) + kLdThreads - 1) / kLdThreads;
+}
+__host__ __device__ constexpr bool ld_reg_fits(int N, int RB)
+{
+    return RB == 2 ? ld_reg_units(N, 2) <= 5 : (RB == 4 || RB == 8) && ld_reg_units(N, RB) <= 3;
+}
+// Window sums join the state in registers up to 6 floats a thread, beyond that
+// they have a place of their own behind the operand.
+__host__ __device__ constexpr bool ld_win_in_regs(int RB, int K)
+{
+    return K * (RB >= 4 ? 4 : 2) <= 6;
+}
+__host__ __device__ constexpr uint32_t ld_reg_bytes(int N, int RB, bool bf16)
+{
+    const int K = ld_reg_units(N, RB);
+    return align16(4u * (uint32_t)(N + 1) * RB * (bf16 ? 2u : 4u)) +
+           (ld_win_in_regs(RB, K) ? 0u : (uint32_t)K * kLdThreads * (RB >= 4 ? 16u : 8u));
+}
+__host__ __device__ constexpr int ld_code(int RB, int K) { return RB * 16 + K; }
+
 struct LdMember {
     const uint2* lists;    // [N] four u16 entries
     const float* h;        // [N] or null
@@ -54,7 +79,7 @@ struct LdMember {
 
 struct LdArgs {
     const LdMember* mem;
-    const int2* items;     // (member, replica block), longest member first
+    const int4* items;     // {member, first replica, ld_code (register form)}, longest first
     int* counter;
     const StepCoef* sched;
     uint32_t* status;
@@ -190,9 +215,9 @@ __global__ void __launch_bounds__(kLdThreads, 1) k_batch_lowdeg(const LdArgs a)
         __syncthreads();
         const int it = s_item;
         if (it >= a.nitems) break;
-        const int2 wi = a.items[it];
+        const int4 wi = a.items[it];
         const LdMember m = a.mem[wi.x];
-        const int N = m.N, NRB = N * RB, rep0 = wi.y * RB;
+        const int N = m.N, NRB = N * RB, rep0 = wi.y;
         const uint32_t buf = (uint32_t)(N + 1) * RB * ES;
         const uint32_t opb = align16(2u * buf);
         const uint32_t master = s0 + opb;
@@ -337,6 +362,252 @@ __global__ void __launch_bounds__(kLdThreads, 1) k_batch_lowdeg(const LdArgs a)
     }
 }
 
+// ---- state in registers -------------------------------------------------------
+// A thread owns the same K units (a spin, PR replicas) of its item at every step,
+// so momentum, window sums, flux and list stay in its registers; shared memory
+// holds the operand alone, with a negated copy of every row ([+ N + 1 rows |
+// - N + 1 rows], two step buffers), so that a list entry is a row number and a
+// gather needs no sign.  k_batch_lowdeg was bound by instructions: per spin and
+// pair about 110, of which the kick needs ten; shared-memory wavefronts came
+// next, a third of them list, momentum and window sums.  96 members of N = 200
+// to 5000 x 64 replicas, 100 steps in FP32, all in the window: 3157 -> 2484 us,
+// the same bits.
+
+template <bool BF16, int PR>
+struct LdVec;                                   // PR replicas of one operand row
+template <> struct LdVec<false, 2> {
+    static __device__ __forceinline__ void load(uint32_t a, uint64_t* v)
+    {
+        const uint2 x = lds64(a);
+        v[0] = (uint64_t)x.x | ((uint64_t)x.y << 32);
+    }
+    static __device__ __forceinline__ void store(uint32_t a, uint32_t an, const uint64_t* v)
+    {
+        const uint2 x = make_uint2((uint32_t)v[0], (uint32_t)(v[0] >> 32));
+        sts64(a, x);
+        sts64(an, make_uint2(x.x ^ 0x80000000u, x.y ^ 0x80000000u));
+    }
+};
+template <> struct LdVec<false, 4> {
+    static __device__ __forceinline__ void load(uint32_t a, uint64_t* v)
+    {
+        asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(a));
+    }
+    static __device__ __forceinline__ void store(uint32_t a, uint32_t an, const uint64_t* v)
+    {
+        constexpr uint64_t sg = 0x8000000080000000ull;
+        asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(a), "l"(v[0]), "l"(v[1]));
+        asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(an), "l"(v[0] ^ sg), "l"(v[1] ^ sg));
+    }
+};
+template <int PR> struct LdVec<true, PR> {
+    static __device__ __forceinline__ void load(uint32_t a, uint64_t* v)
+    {
+        uint32_t x[PR / 2];
+        if constexpr (PR == 2) {
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x[0]) : "r"(a));
+        } else {
+            const uint2 w = lds64(a);
+            x[0] = w.x;
+            x[PR / 2 - 1] = w.y;
+        }
+#pragma unroll
+        for (int c = 0; c < PR / 2; ++c)
+            v[c] = (uint64_t)(x[c] << 16) | ((uint64_t)(x[c] & 0xffff0000u) << 32);
+    }
+    static __device__ __forceinline__ void store(uint32_t a, uint32_t an, const uint64_t* v)
+    {
+        uint32_t x[PR / 2];
+#pragma unroll
+        for (int c = 0; c < PR / 2; ++c) {
+            const __nv_bfloat162 b = __floats2bfloat162_rn(lo(v[c]), hi(v[c]));
+            x[c] = *reinterpret_cast<const uint32_t*>(&b);
+        }
+        if constexpr (PR == 2) {
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(x[0]));
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(an), "r"(x[0] ^ 0x80008000u));
+        } else {
+            sts64(a, make_uint2(x[0], x[PR / 2 - 1]));
+            sts64(an, make_uint2(x[0] ^ 0x80008000u, x[PR / 2 - 1] ^ 0x80008000u));
+        }
+    }
+};
+
+// One work item: RB replicas of member m from rep0 on, for the whole run.  The
+// arithmetic is k_batch_lowdeg's at M = 6, operation by operation.
+template <int RB, bool BF16, int K>
+__device__ __forceinline__ void ld_item(const LdArgs& a, const LdMember& m, int rep0, uint32_t s0)
+{
+    constexpr uint32_t ROW = RB * (BF16 ? 2u : 4u);   // bytes of an operand row
+    constexpr int PR = RB >= 4 ? 4 : 2, TR = RB / PR, NP = PR / 2;
+    using V = LdVec<BF16, PR>;
+    const int t = threadIdx.x, N = m.N, U = N * TR;
+    const uint32_t half = (uint32_t)(N + 1) * ROW, buf = 2u * half;
+    const int row0 = t / TR, r0 = (t % TR) * PR;      // unit k: row0 + k * RSTEP, r0
+    constexpr int RSTEP = kLdThreads / TR;
+    const uint32_t lane = (uint32_t)r0 * (BF16 ? 2u : 4u);
+    const uint32_t own = lane + (uint32_t)row0 * ROW;
+
+    // row N of the + halves is the lists' padding: zero in both step buffers
+    if (t < 2 * (int)(ROW / 4u))
+        sts32(s0 + (t & 1) * buf + (uint32_t)N * ROW + (uint32_t)(t >> 1) * 4u, 0.f);
+    uint2 li[K];
+    constexpr bool WREG = ld_win_in_regs(RB, K);
+    const uint32_t sw = s0 + align16(2u * buf) + (uint32_t)t * 8u;   // window sums, else
+    constexpr bool FREG = BF16 || K * PR <= 8;   // FP32 flux, else read back from the operand
+    uint64_t f[K][NP], p[K][NP], w[WREG ? K : 1][NP];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        li[k] = make_uint2(0u, 0u);
+#pragma unroll
+        for (int c = 0; c < NP; ++c) {
+            f[k][c] = p[k][c] = 0ull;
+            if constexpr (WREG) w[k][c] = 0ull;
+            else sts64(sw + (uint32_t)((k * NP + c) * kLdThreads * 8), make_uint2(0u, 0u));
+        }
+        const int row = row0 + k * RSTEP;
+        if (t + k * kLdThreads >= U) continue;
+        const uint2 l = __ldg(m.lists + row);
+        const uint32_t neg = (uint32_t)(N + 1);
+        // bit 15 set -> the row of the negated half
+        const uint32_t e0 = (l.x & 0x7fffu) + ((l.x & 0x8000u) ? neg : 0u);
+        const uint32_t e1 = ((l.x >> 16) & 0x7fffu) + ((l.x >> 31) ? neg : 0u);
+        const uint32_t e2 = (l.y & 0x7fffu) + ((l.y & 0x8000u) ? neg : 0u);
+        const uint32_t e3 = ((l.y >> 16) & 0x7fffu) + ((l.y >> 31) ? neg : 0u);
+        li[k] = make_uint2(e0 | (e1 << 16), e2 | (e3 << 16));
+        float x[PR], q[PR];
+#pragma unroll
+        for (int i = 0; i < PR; ++i) {
+            const int rep = rep0 + r0 + i;
+            x[i] = q[i] = 0.f;
+            if (rep >= a.R) continue;
+            if (a.init == HQA_INIT_GIVEN) {
+                x[i] = m.phi0[(size_t)rep * N + row];
+                q[i] = m.p0[(size_t)rep * N + row];
+            } else {
+                const uint64_t c = ((uint64_t)rep << 32) | (uint64_t)row;
+                q[i] = (ld_splitmix(m.seed, c) >> 63) ? -1.f : 1.f;
+                if (a.init == HQA_INIT_RANDOM_FLUX) {
+                    const uint64_t z = ld_splitmix(m.seed, c | (1ull << 62));
+                    x[i] = (float)((int64_t)(z >> 40) - (1 << 23)) * 0x1p-26f;
+                }
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NP; ++c) {
+            f[k][c] = pk(x[2 * c], x[2 * c + 1]);
+            p[k][c] = pk(q[2 * c], q[2 * c + 1]);
+        }
+        const uint32_t o = s0 + own + (uint32_t)(k * RSTEP) * ROW;
+        V::store(o, o + half, f[k]);
+    }
+    __syncthreads();
+
+    const int64_t win0 = a.S - (int64_t)a.W;   // steps j >= win0 add phi^(j+1) to the window
+    uint32_t cur = s0, nxt = s0 + buf;
+    for (int64_t j = 0; j < a.S; ++j) {
+        const float4 cf = __ldg(reinterpret_cast<const float4*>(a.sched) + j);
+        const uint64_t kA = pk(cf.x, cf.x), kB = pk(cf.y, cf.y), dA = pk(cf.z, cf.z);
+        const bool in_win = j >= win0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (k == K - 1 && t + k * kLdThreads >= U) continue;
+            uint64_t v0[NP], v1[NP], v2[NP], v3[NP];
+            V::load(cur + lane + (li[k].x & 0xffffu) * ROW, v0);
+            V::load(cur + lane + (li[k].x >> 16) * ROW, v1);
+            V::load(cur + lane + (li[k].y & 0xffffu) * ROW, v2);
+            V::load(cur + lane + (li[k].y >> 16) * ROW, v3);
+            if constexpr (!FREG) V::load(cur + own + (uint32_t)(k * RSTEP) * ROW, f[k]);
+#pragma unroll
+            for (int c = 0; c < NP; ++c) {
+                const uint64_t L = add2(add2(v0[c], v1[c]), add2(v2[c], v3[c]));
+                const uint64_t f2 = mul2(f[k][c], f[k][c]);
+                const uint64_t pw = mul2(mul2(f[k][c], f2), f2);
+                p[k][c] = sub2(p[k][c], fma2(kA, pw, mul2(kB, L)));
+                f[k][c] = fma2(dA, p[k][c], f[k][c]);
+            }
+            const uint32_t o = nxt + own + (uint32_t)(k * RSTEP) * ROW;
+            V::store(o, o + half, f[k]);
+            if (in_win) {
+#pragma unroll
+                for (int c = 0; c < NP; ++c) {
+                    if constexpr (WREG) {
+                        w[k][c] = add2(w[k][c], f[k][c]);
+                    } else {
+                        const uint32_t q = sw + (uint32_t)((k * NP + c) * kLdThreads * 8);
+                        const uint2 x = lds64(q);
+                        const uint64_t y = add2((uint64_t)x.x | ((uint64_t)x.y << 32), f[k][c]);
+                        sts64(q, make_uint2((uint32_t)y, (uint32_t)(y >> 32)));
+                    }
+                }
+            }
+        }
+        const uint32_t x = cur;
+        cur = nxt;
+        nxt = x;
+        __syncthreads();
+    }
+
+    // outputs, [R][N] member block, coalesced over spins
+    const float inv_w = 1.0f / (float)(a.S < a.W ? a.S : (int64_t)a.W);
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        if (t + k * kLdThreads >= U) continue;
+        if constexpr (!FREG) V::load(cur + own + (uint32_t)(k * RSTEP) * ROW, f[k]);
+#pragma unroll
+        for (int i = 0; i < PR; ++i) {
+            const int rep = rep0 + r0 + i;
+            if (rep >= a.R) continue;
+            const float x = (i & 1) ? hi(f[k][i / 2]) : lo(f[k][i / 2]);
+            const float q = (i & 1) ? hi(p[k][i / 2]) : lo(p[k][i / 2]);
+            const size_t o = (size_t)rep * N + row0 + k * RSTEP;
+            if (m.phi_out) m.phi_out[o] = x;
+            if (m.p_out) m.p_out[o] = q;
+            if (m.phibar_out) {
+                float y;
+                if constexpr (WREG) y = (i & 1) ? hi(w[k][i / 2]) : lo(w[k][i / 2]);
+                else y = lds32(sw + (uint32_t)((k * NP + i / 2) * kLdThreads * 8 + (i & 1) * 4));
+                m.phibar_out[o] = y * inv_w;
+            }
+            bad |= !(isfinite(x) && isfinite(q));
+        }
+    }
+    if (__syncthreads_or(bad) && t == 0) atomicOr(a.status, HQA_DEV_NONFINITE);
+}
+
+template <bool BF16>
+__global__ void __launch_bounds__(kLdThreads, 1) k_batch_lowdeg_reg(const LdArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_item;
+    const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = atomicAdd(a.counter, 1);
+        __syncthreads();
+        const int it = s_item;
+        if (it >= a.nitems) break;
+        const int4 wi = a.items[it];
+        const LdMember m = a.mem[wi.x];
+        const int rep0 = wi.y;
+        switch (wi.z) {
+        case ld_code(2, 1): ld_item<2, BF16, 1>(a, m, rep0, s0); break;
+        case ld_code(2, 2): ld_item<2, BF16, 2>(a, m, rep0, s0); break;
+        case ld_code(2, 3): ld_item<2, BF16, 3>(a, m, rep0, s0); break;
+        case ld_code(2, 4): ld_item<2, BF16, 4>(a, m, rep0, s0); break;
+        case ld_code(2, 5): ld_item<2, BF16, 5>(a, m, rep0, s0); break;
+        case ld_code(4, 1): ld_item<4, BF16, 1>(a, m, rep0, s0); break;
+        case ld_code(4, 2): ld_item<4, BF16, 2>(a, m, rep0, s0); break;
+        case ld_code(4, 3): ld_item<4, BF16, 3>(a, m, rep0, s0); break;
+        case ld_code(8, 1): ld_item<8, BF16, 1>(a, m, rep0, s0); break;
+        case ld_code(8, 2): ld_item<8, BF16, 2>(a, m, rep0, s0); break;
+        case ld_code(8, 3): ld_item<8, BF16, 3>(a, m, rep0, s0); break;
+        default: break;
+        }
+    }
+}
+
 template <int RB, bool BF16>
 cudaError_t launch_ld(const LdArgs& a, int grid, size_t smem, cudaStream_t st)
 {
@@ -344,6 +615,53 @@ cudaError_t launch_ld(const LdArgs& a, int grid, size_t smem, cudaStream_t st)
     if (e != cudaSuccess) return e;
     k_batch_lowdeg<RB, BF16><<<grid, kLdThreads, smem, st>>>(a);
     return cudaGetLastError();
+}
+
+template <bool BF16>
+cudaError_t launch_ld_reg(const LdArgs& a, int grid, size_t smem, cudaStream_t st)
+{
+    const cudaError_t e = hqa_smem_attr((const void*)k_batch_lowdeg_reg<BF16>, smem);
+    if (e != cudaSuccess) return e;
+    k_batch_lowdeg_reg<BF16><<<grid, kLdThreads, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+// Whether the register form can run a launch of blocking RB (it also needs the
+// paper's M = 6), and each member's blocking in it (`mrb`).  No field, at least two
+// replicas a thread, and every member within its units per thread; a single
+// replica per item (RB = 1, few items) stays with k_batch_lowdeg.  Where the
+// caller left the blocking open, small members take 4 or 8 replicas per item,
+// smallest first: a list entry then serves more replicas and a step's barrier
+// more work.  No item grows beyond the longest that the launch has anyway, and
+// at least four items per SM are left to balance the queue.  Depends on members,
+// R and RB alone, so that a table uploaded for one run serves a captured one of
+// another precision or M.
+bool ld_reg_blocking(const hqa_ctx* b, int RB, int32_t R, std::vector<int>& mrb)
+{
+    const int count = (int)b->members.size();
+    mrb.assign(count, RB);
+    if (RB < 2) return false;
+    int64_t longest = 0, items = 0;
+    for (const hqa_ctx* m : b->members) {
+        if (m->has_h || !ld_reg_fits(m->N, RB)) return false;
+        longest = std::max<int64_t>(longest, (int64_t)m->N * RB);
+        items += (R + RB - 1) / RB;
+    }
+    std::vector<int> order(count);
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int x, int y) { return b->members[x]->N < b->members[y]->N; });
+    for (int k : order) {
+        const int N = b->members[k]->N;
+        for (int rb = 2 * RB; rb <= 8 && rb <= R; rb *= 2) {
+            const int64_t left = items - (R + mrb[k] - 1) / mrb[k] + (R + rb - 1) / rb;
+            if ((int64_t)N * rb > longest || !ld_reg_fits(N, rb) || left < 4 * (int64_t)b->sm_count)
+                break;
+            items = left;
+            mrb[k] = rb;
+        }
+    }
+    return true;
 }
 
 }  // namespace
@@ -390,13 +708,24 @@ int hqa_lowdeg_pick_rb(const hqa_ctx* b, int32_t R, int prec)
 hqa_status hqa_lowdeg_launch_md(hqa_ctx* b, int RB, int prec, const StepCoef* d_sched, int64_t S,
                                 int32_t W, int32_t R, uint64_t seed, int init, const float* phi0,
                                 const float* p0, int M, float* phi_out, float* p_out,
-                                float* phibar_out, cudaStream_t st)
+                                float* phibar_out, bool raise, cudaStream_t st)
 {
     if (!hqa_lowdeg_eligible(b) || prec == HQA_PREC_BF16X2) return HQA_ERR_UNSUPPORTED;
     if (RB != 1 && RB != 2 && RB != 4) return HQA_ERR_UNSUPPORTED;
-    const size_t smem = hqa_lowdeg_smem_bytes(b, RB, prec);
+    size_t smem = hqa_lowdeg_smem_bytes(b, RB, prec);
     if (smem > b->smem_optin - 1024) return HQA_ERR_TOO_LARGE;
     const int count = (int)b->members.size();
+    const bool bf = prec == HQA_PREC_BF16;
+    std::vector<int> mrb;
+    const bool can_reg = ld_reg_blocking(b, RB, R, mrb);
+    bool reg = can_reg && M == 6;
+    if (reg) {
+        size_t need = 0;
+        for (int k = 0; k < count; ++k)
+            need = std::max<size_t>(need, ld_reg_bytes(b->members[k]->N, raise ? mrb[k] : RB, bf));
+        reg = need <= b->smem_optin - 1024;
+        if (reg) smem = need;
+    }
     // compact lists of every member, built once (outside any capture)
     if (b->ld_off.empty()) {
         if (hqa_capturing()) return hqa_capture_note(HQA_ERR_UNSUPPORTED);
@@ -421,8 +750,6 @@ hqa_status hqa_lowdeg_launch_md(hqa_ctx* b, int RB, int prec, const StepCoef* d_
         b->ld_off = off;
     }
     std::vector<LdMember> mem(count);
-    std::vector<int2> items;
-    const int blocks = (R + RB - 1) / RB;
     for (int k = 0; k < count; ++k) {
         const hqa_ctx* m = b->members[k];
         LdMember x;
@@ -438,14 +765,28 @@ hqa_status hqa_lowdeg_launch_md(hqa_ctx* b, int RB, int prec, const StepCoef* d_
         x.seed = seed + (uint64_t)(k + 1) * 0x632BE59BD9B4E019ull;
         x.N = m->N;
         mem[k] = x;
-        for (int blk = 0; blk < blocks; ++blk) items.push_back(make_int2(k, blk));
     }
-    // longest member first (ties in member order)
-    std::stable_sort(items.begin(), items.end(), [&](const int2& x, const int2& y) {
-        return b->members[x.x]->N > b->members[y.x]->N;
-    });
+    // two tables: every member at RB, and each at its own blocking (register form,
+    // blocking left open); most work first, ties in member order
+    auto fill = [&](const std::vector<int>& rbs) {
+        std::vector<int4> v;
+        for (int k = 0; k < count; ++k) {
+            const int code = can_reg ? ld_code(rbs[k], ld_reg_units(b->members[k]->N, rbs[k])) : 0;
+            for (int rep = 0; rep < R; rep += rbs[k]) v.push_back(make_int4(k, rep, code, 0));
+        }
+        std::stable_sort(v.begin(), v.end(), [&](const int4& x, const int4& y) {
+            return (int64_t)b->members[x.x]->N * rbs[x.x] > (int64_t)b->members[y.x]->N * rbs[y.x];
+        });
+        return v;
+    };
+    std::vector<int4> items = fill(std::vector<int>(count, RB));
+    const size_t even = items.size();
+    if (can_reg) {
+        const std::vector<int4> v = fill(mrb);
+        items.insert(items.end(), v.begin(), v.end());
+    }
     const size_t off_items = (mem.size() * sizeof(LdMember) + 255) & ~(size_t)255;
-    const size_t off_cnt = off_items + ((items.size() * sizeof(int2) + 255) & ~(size_t)255);
+    const size_t off_cnt = off_items + ((items.size() * sizeof(int4) + 255) & ~(size_t)255);
     void* const held = b->d_ldwork;
     hqa_status s = hqa_reserve(b, &b->d_ldwork, &b->ldwork_cap, off_cnt + 256);
     if (s != HQA_OK) return s;
@@ -457,7 +798,7 @@ hqa_status hqa_lowdeg_launch_md(hqa_ctx* b, int RB, int prec, const StepCoef* d_
     const char* mb = reinterpret_cast<const char*>(mem.data());
     const char* ib = reinterpret_cast<const char*>(items.data());
     std::copy(mb, mb + mem.size() * sizeof(LdMember), tab.begin());
-    std::copy(ib, ib + items.size() * sizeof(int2), tab.begin() + (std::ptrdiff_t)off_items);
+    std::copy(ib, ib + items.size() * sizeof(int4), tab.begin() + (std::ptrdiff_t)off_items);
     if (tab != b->ldwork_host) {
         if (hqa_capturing()) return hqa_capture_note(HQA_ERR_UNSUPPORTED);
         ++b->generation;
@@ -469,19 +810,19 @@ hqa_status hqa_lowdeg_launch_md(hqa_ctx* b, int RB, int prec, const StepCoef* d_
     HQA_CUDA_TRY(cudaMemsetAsync(w + off_cnt, 0, sizeof(int), st));
     LdArgs a;
     a.mem = reinterpret_cast<const LdMember*>(w);
-    a.items = reinterpret_cast<const int2*>(w + off_items);
+    a.items = reinterpret_cast<const int4*>(w + off_items) + (reg && raise ? even : 0);
     a.counter = reinterpret_cast<int*>(w + off_cnt);
     a.sched = d_sched;
     a.status = b->d_status;
     a.S = S;
-    a.nitems = (int)items.size();
+    a.nitems = (int)(reg && raise ? items.size() - even : even);
     a.W = W;
     a.R = R;
     a.M = M;
     a.init = init;
-    const bool bf = prec == HQA_PREC_BF16;
     cudaError_t e;
-    if (RB == 4) e = bf ? launch_ld<4, true>(a, b->sm_count, smem, st) : launch_ld<4, false>(a, b->sm_count, smem, st);
+    if (reg) e = bf ? launch_ld_reg<true>(a, b->sm_count, smem, st) : launch_ld_reg<false>(a, b->sm_count, smem, st);
+    else if (RB == 4) e = bf ? launch_ld<4, true>(a, b->sm_count, smem, st) : launch_ld<4, false>(a, b->sm_count, smem, st);
     else if (RB == 2) e = bf ? launch_ld<2, true>(a, b->sm_count, smem, st) : launch_ld<2, false>(a, b->sm_count, smem, st);
     else e = bf ? launch_ld<1, true>(a, b->sm_count, smem, st) : launch_ld<1, false>(a, b->sm_count, smem, st);
     return e == cudaSuccess ? HQA_OK : HQA_ERR_CUDA;

@@ -277,10 +277,11 @@ int hqa_sparse_pick_rb(const hqa_ctx* ctx, int32_t R, int prec);
 bool hqa_lowdeg_eligible(const hqa_ctx* batch);
 size_t hqa_lowdeg_smem_bytes(const hqa_ctx* batch, int RB, int prec);
 int hqa_lowdeg_pick_rb(const hqa_ctx* batch, int32_t R, int prec);
+// raise: the blocking was left open, so small members may take a larger one
 hqa_status hqa_lowdeg_launch_md(hqa_ctx* batch, int RB, int prec, const StepCoef* d_sched,
                                 int64_t S, int32_t W, int32_t R, uint64_t seed, int init,
                                 const float* phi0, const float* p0, int M, float* phi_out,
-                                float* p_out, float* phibar_out, cudaStream_t st);
+                                float* p_out, float* phibar_out, bool raise, cudaStream_t st);
 size_t hqa_sparse_smem_bytes(const hqa_ctx* ctx, int RB, int prec);
 hqa_status hqa_sparse_launch_md(hqa_ctx* ctx, const SparsePlan* plan, const StepCoef* d_sched,
                                 int64_t S, int32_t W, int32_t R, uint64_t seed, int init,
