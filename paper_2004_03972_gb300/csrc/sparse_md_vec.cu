@@ -19,13 +19,16 @@
 //     memory once per launch, 8 positions per 128-bit load;
 //   * sums use Blackwell's packed FP32 add (add.rn.f32x2);
 //   * tuples are assigned to warps on the host (longest-processing-time
-//     first); one __syncthreads() per leapfrog step; window sums live in
-//     global memory (touched only in the last W steps);
+//     first); one __syncthreads() per leapfrog step;
 //   * a lane updates the same rows at every step (the tuple-to-warp map is
 //     fixed for the launch), so when no warp owns more than four tuples
 //     the FP32 flux and momentum of the lane's rows stay in its
 //     registers for the whole trajectory: the kick reads no shared memory
-//     and writes only the next operand buffer.
+//     and writes only the next operand buffer; the window sums of the last
+//     W steps then take the momenta's shared memory (in global memory a step
+//     waited for them: ER N = 800 x 1024, 200 steps in FP32, half of them in the
+//     window, 1259 -> 1228 us, BF16, 100 steps, 425 -> 421 us), else they live in
+//     global memory.  Loading a list chunk one chunk ahead cost 1 %.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -236,7 +239,7 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
     const uint32_t master = op0 + 2u * buf_bytes;
     const uint32_t ps = master + (BF16 ? (uint32_t)a.Npad * RB * 4u : 0u);
     const int NRB = a.N * RB;
-    float* gw = a.gwin + (size_t)blockIdx.x * a.Npad * RB;
+    float* gw = REG > 0 ? nullptr : a.gwin + (size_t)blockIdx.x * a.Npad * RB;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane / LPR, q = lane % LPR;
@@ -247,7 +250,8 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
         sts128(s0 + o, __ldg(a.entries + o / 16u));
     for (uint32_t o = threadIdx.x * 16u; o < 2u * buf_bytes; o += blockDim.x * 16u)
         sts128(op0 + o, make_uint4(0, 0, 0, 0));
-    for (int o = threadIdx.x; o < a.Npad * RB; o += blockDim.x) gw[o] = 0.f;
+    if constexpr (REG == 0)
+        for (int o = threadIdx.x; o < a.Npad * RB; o += blockDim.x) gw[o] = 0.f;
     __syncthreads();
     for (int idx = threadIdx.x; idx < NRB; idx += blockDim.x) {
         const int row = idx / RB, rr = idx % RB, rep = rep0 + rr;
@@ -278,6 +282,7 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
     }
     __syncthreads();
 
+    const uint32_t dead = op0 + (uint32_t)((a.S & 1) ^ 1) * buf_bytes;   // after the last step
     const int wbeg = __ldg(a.warp_off + warp), wend = __ldg(a.warp_off + warp + 1);
     const int64_t win0 = a.S - (int64_t)a.W;
     const int mhalf = (a.M - 2) / 2;
@@ -315,6 +320,8 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
                 if (rok[kk]) {
                     x = lds128((BF16 ? master : op0) + (re0[kk] + 4 * k4) * 4u);
                     y = lds128(ps + (re0[kk] + 4 * k4) * 4u);
+                    // from here to the end of the run ps holds the window sums
+                    sts128(ps + (re0[kk] + 4 * k4) * 4u, make_uint4(0, 0, 0, 0));
                 }
                 rphi[kk][4 * k4] = __uint_as_float(x.x); rphi[kk][4 * k4 + 1] = __uint_as_float(x.y);
                 rphi[kk][4 * k4 + 2] = __uint_as_float(x.z); rphi[kk][4 * k4 + 3] = __uint_as_float(x.w);
@@ -371,17 +378,19 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
                 if (in_win) {
 #pragma unroll
                     for (int k4 = 0; k4 < V / 4; ++k4) {
-                        float4* wp = reinterpret_cast<float4*>(gw + re0[kk] + 4 * k4);
-                        float4 w = *wp;
-                        w.x += rphi[kk][4 * k4]; w.y += rphi[kk][4 * k4 + 1];
-                        w.z += rphi[kk][4 * k4 + 2]; w.w += rphi[kk][4 * k4 + 3];
-                        *wp = w;
+                        const uint32_t o = ps + (re0[kk] + 4 * k4) * 4u;
+                        const uint4 w = lds128(o);
+                        sts128(o, make_uint4(__float_as_uint(__uint_as_float(w.x) + rphi[kk][4 * k4]),
+                                             __float_as_uint(__uint_as_float(w.y) + rphi[kk][4 * k4 + 1]),
+                                             __float_as_uint(__uint_as_float(w.z) + rphi[kk][4 * k4 + 2]),
+                                             __float_as_uint(__uint_as_float(w.w) + rphi[kk][4 * k4 + 3])));
                     }
                 }
             }
             __syncthreads();
         }
-        // final state back to the shared layout the output code reads
+        // final state back to the shared layout the output code reads; the window
+        // sums move to the operand buffer that no step reads any more
         const uint32_t fin = op0 + (uint32_t)(a.S & 1) * buf_bytes;
 #pragma unroll
         for (int kk = 0; kk < RS; ++kk) {
@@ -389,6 +398,7 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
 #pragma unroll
             for (int k4 = 0; k4 < V / 4; ++k4) {
                 const uint32_t o = (re0[kk] + 4 * k4) * 4u;
+                sts128(dead + o, lds128(ps + o));
                 sts128(ps + o, make_uint4(__float_as_uint(rp[kk][4 * k4]), __float_as_uint(rp[kk][4 * k4 + 1]),
                                           __float_as_uint(rp[kk][4 * k4 + 2]),
                                           __float_as_uint(rp[kk][4 * k4 + 3])));
@@ -493,7 +503,9 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
         float phi, p;
         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(phi) : "r"((BF16 ? master : fin) + e * 4u));
         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(p) : "r"(ps + e * 4u));
-        const float w = gw[e];
+        float w;
+        if constexpr (REG > 0) asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w) : "r"(dead + e * 4u));
+        else w = gw[e];
         const size_t o = (size_t)rep * a.N + row;
         if (a.phi_out) a.phi_out[o] = phi;
         if (a.p_out) a.p_out[o] = p;
@@ -1041,9 +1053,6 @@ hqa_status hqa_vec_launch_md(hqa_ctx* ctx, const SparsePlan* pl, const StepCoef*
     const size_t smem = hqa_vec_smem_bytes(ctx, pl->RB, pl->prec, pl->ent_bytes);
     if (smem > ctx->smem_optin) return HQA_ERR_TOO_LARGE;
     const int blocks = (R + pl->RB - 1) / pl->RB;
-    hqa_status s = hqa_reserve(ctx, &ctx->d_state, &ctx->state_cap,
-                               (size_t)blocks * pl->Npad * pl->RB * sizeof(float));
-    if (s != HQA_OK) return s;
     VArgs a = common_args(ctx, pl, R);
     a.sched = d_sched;
     a.phi0 = phi0;
@@ -1051,11 +1060,16 @@ hqa_status hqa_vec_launch_md(hqa_ctx* ctx, const SparsePlan* pl, const StepCoef*
     a.phi_out = phi_out;
     a.p_out = p_out;
     a.phibar_out = phibar_out;
-    a.gwin = static_cast<float*>(ctx->d_state);
     a.reg = 0;
     for (int r : {1, 2, 4})
         if (a.reg == 0 && pl->max_wt <= r && pl->NW * 32 <= reg_threads(r, pl->prec == HQA_PREC_BF16))
             a.reg = r;
+    if (a.reg == 0) {   // window sums in global memory
+        hqa_status s = hqa_reserve(ctx, &ctx->d_state, &ctx->state_cap,
+                                   (size_t)blocks * pl->Npad * pl->RB * sizeof(float));
+        if (s != HQA_OK) return s;
+        a.gwin = static_cast<float*>(ctx->d_state);
+    }
     a.seed = seed;
     a.S = S;
     a.W = W;
