@@ -284,16 +284,28 @@ hqa_status choose_plan(hqa_ctx* ctx, int32_t R, const hqa_run_opts& opts, const 
             o.replicas_per_block = it->second.second;
         }
     }
+    // A full 16-byte vector of replicas per lane, or half of one where that still
+    // gives every block an SM of its own.  A step's time is that of its block's
+    // gathers, so idle SMs are worth more than wide loads: ER N = 800 x 300, 100
+    // steps, FP32 381 -> 238 us, BF16 423 -> 269 us; N = 1000 of mean degree 8 x 256
+    // 141 -> 99 and 197 -> 122 us.  Only where the blocking is left open; a stated or
+    // tuned one is taken as it is.
+    const int V = o.precision == HQA_PREC_BF16 ? 8 : 4;
+    const bool half_fits = R >= V && (R + V / 2 - 1) / (V / 2) <= ctx->sm_count &&
+                           hqa_vec_supported(ctx, V / 2, o.precision);
     int RB = o.replicas_per_block;
     int rb_scalar = RB;   // the scalar kernel's blocking if the vectorised one is not used
+    bool narrow = false;
     if (RB == 0) {
         RB = rb_scalar = hqa_sparse_pick_rb(ctx, R, o.precision);
-        // the vectorised kernel needs a full 16-byte vector of replicas per lane
-        const int V = o.precision == HQA_PREC_BF16 ? 8 : 4;
-        if (o.kernel != HQA_KERNEL_SCALAR && RB < V && RB > 0 && R >= V) RB = V;
+        if (o.kernel != HQA_KERNEL_SCALAR && RB < V && RB > 0 && R >= V) {
+            RB = V;
+            narrow = half_fits;
+        }
     }
     if (RB == 0) return HQA_ERR_TOO_LARGE;
-    if (o.kernel != HQA_KERNEL_SCALAR && hqa_vec_supported(ctx, RB, o.precision)) {
+    if (narrow) RB = V / 2;
+    if (o.kernel != HQA_KERNEL_SCALAR && (narrow || RB >= V) && hqa_vec_supported(ctx, RB, o.precision)) {
         const SparsePlan* vp = nullptr;
         hqa_status s = hqa_vec_plan(ctx, RB, o.precision, &vp);
         if (s != HQA_OK) return s;

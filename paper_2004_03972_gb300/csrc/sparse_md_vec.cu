@@ -6,6 +6,8 @@
 //   * every lane gathers 16 bytes per neighbour -- V = 4 FP32 or V = 8 BF16
 //     replicas -- with one 128-bit shared load, so a warp reads G rows x RB
 //     replicas per instruction (G = 32 * V / RB);
+//     (or 8 bytes, V = 2 or 4, in two 16-lane phases, where few replicas would
+//     leave SMs idle: see choose_plan);
 //   * the operand keeps phi and -phi ([+ slots | - slots]) so a coupling of
 //     -1 is a gather from the negated copy: every position is a plain add;
 //   * a 128-bit shared load is served in four 8-lane phases, each covering P
@@ -50,6 +52,13 @@ __host__ __device__ constexpr int reg_threads(int reg, bool bf16)
     return reg == 1 ? (bf16 ? 896 : 1024) : reg == 2 ? (bf16 ? 704 : 832) : 512;
 }
 
+// Replicas per lane: 16-byte gathers, or 8-byte ones at half that many replicas.
+__host__ __device__ constexpr int vec_of(int RB, bool bf16)
+{
+    const int V = bf16 ? 8 : 4;
+    return RB < V ? V / 2 : V;
+}
+
 __device__ __forceinline__ uint64_t smix(uint64_t seed, uint64_t counter)
 {
     // SplitMix64 (Steele, Lea, Flood 2014): output number counter+1 of the stream.
@@ -71,6 +80,75 @@ __device__ __forceinline__ void sts128(uint32_t a, uint4 v)
 {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y),
                  "r"(v.z), "r"(v.w));
+}
+
+__device__ __forceinline__ uint2 lds64(uint32_t a)
+{
+    uint2 v;
+    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
+
+__device__ __forceinline__ void sts64(uint32_t a, uint2 v)
+{
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y));
+}
+
+// V floats of shared memory (16-byte accesses, 8 bytes at V = 2)
+template <int V>
+__device__ __forceinline__ void lds_state(uint32_t a, float* x)
+{
+    if constexpr (V == 2) {
+        const uint2 v = lds64(a);
+        x[0] = __uint_as_float(v.x);
+        x[1] = __uint_as_float(v.y);
+    } else {
+#pragma unroll
+        for (int k = 0; k < V; k += 4) {
+            const uint4 v = lds128(a + k * 4u);
+            x[k] = __uint_as_float(v.x);
+            x[k + 1] = __uint_as_float(v.y);
+            x[k + 2] = __uint_as_float(v.z);
+            x[k + 3] = __uint_as_float(v.w);
+        }
+    }
+}
+
+template <int V>
+__device__ __forceinline__ void sts_state(uint32_t a, const float* x)
+{
+    if constexpr (V == 2) {
+        sts64(a, make_uint2(__float_as_uint(x[0]), __float_as_uint(x[1])));
+    } else {
+#pragma unroll
+        for (int k = 0; k < V; k += 4)
+            sts128(a + k * 4u, make_uint4(__float_as_uint(x[k]), __float_as_uint(x[k + 1]),
+                                          __float_as_uint(x[k + 2]), __float_as_uint(x[k + 3])));
+    }
+}
+
+// NW 32-bit words of the operand (2 or 4)
+template <int NW>
+__device__ __forceinline__ void lds_words(uint32_t a, uint32_t* w)
+{
+    if constexpr (NW == 2) {
+        const uint2 v = lds64(a);
+        w[0] = v.x;
+        w[1] = v.y;
+    } else {
+        const uint4 v = lds128(a);
+        w[0] = v.x;
+        w[1] = v.y;
+        w[2] = v.z;
+        w[NW - 1] = v.w;
+    }
+}
+
+template <int NW>
+__device__ __forceinline__ void sts_words(uint32_t a, const uint32_t* w)
+{
+    if constexpr (NW == 2) sts64(a, make_uint2(w[0], w[1]));
+    else sts128(a, make_uint4(w[0], w[1], w[2], w[NW - 1]));
 }
 
 __device__ __forceinline__ void sts32(uint32_t a, float v)
@@ -106,26 +184,6 @@ __device__ __forceinline__ unsigned short bf16_bits(float x)
     return *reinterpret_cast<unsigned short*>(&b);
 }
 
-// One 16-byte gather as NP = V/2 packed f32x2 values.
-template <bool BF16>
-struct Gather {
-    static constexpr int NP = BF16 ? 4 : 2;
-    uint64_t v[NP];
-    __device__ __forceinline__ void load(uint32_t addr)
-    {
-        const uint4 w = lds128(addr);
-        if constexpr (BF16) {
-            // bf16 pair (lo = replica 2k, hi = replica 2k+1) -> two FP32
-            const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) v[k] = pack2(ws[k] << 16, ws[k] & 0xffff0000u);
-        } else {
-            v[0] = pack2(w.x, w.y);
-            v[1] = pack2(w.z, w.w);
-        }
-    }
-};
-
 // Neighbour sum of one tuple for this lane.  ent: shared address of this
 // lane's first uint4 of entries (8 u16 offsets), consecutive chunks G * 16
 // bytes apart; nhalf: number of 4-position half-chunks; base: shared address
@@ -139,57 +197,91 @@ __device__ __forceinline__ void add_bf16x2(float& a0, float& a1, uint32_t w)
         : "+f"(a0), "+f"(a1) : "r"(w));
 }
 
-// BF16 operand: 8 FP32 accumulators, one per replica of the lane.
-template <int G>
+// BF16 operand: V FP32 accumulators, one per replica of the lane.
+template <int G, int V>
 __device__ __forceinline__ void tuple_field_bf16(uint32_t ent, int nhalf, uint32_t base, float* acc)
 {
+    constexpr int SH = V == 8 ? 4 : 3;   // log2 bytes of a gather
 #pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+    for (int k = 0; k < V; ++k) acc[k] = 0.f;
     for (int hc = 0; hc < nhalf; hc += 2) {
         const uint4 e = lds128(ent + (uint32_t)(hc >> 1) * (G * 16u));
         const uint32_t ew[4] = {e.x, e.y, e.z, e.w};
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (h == 1 && hc + 1 >= nhalf) break;
-            uint4 v[4];
-            v[0] = lds128(base + ((ew[2 * h] & 0xffffu) << 4));
-            v[1] = lds128(base + ((ew[2 * h] >> 16) << 4));
-            v[2] = lds128(base + ((ew[2 * h + 1] & 0xffffu) << 4));
-            v[3] = lds128(base + ((ew[2 * h + 1] >> 16) << 4));
+            uint32_t v[4][V / 2];
+            lds_words<V / 2>(base + ((ew[2 * h] & 0xffffu) << SH), v[0]);
+            lds_words<V / 2>(base + ((ew[2 * h] >> 16) << SH), v[1]);
+            lds_words<V / 2>(base + ((ew[2 * h + 1] & 0xffffu) << SH), v[2]);
+            lds_words<V / 2>(base + ((ew[2 * h + 1] >> 16) << SH), v[3]);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                add_bf16x2(acc[0], acc[1], v[u].x);
-                add_bf16x2(acc[2], acc[3], v[u].y);
-                add_bf16x2(acc[4], acc[5], v[u].z);
-                add_bf16x2(acc[6], acc[7], v[u].w);
-            }
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int k = 0; k < V / 2; ++k) add_bf16x2(acc[2 * k], acc[2 * k + 1], v[u][k]);
         }
     }
 }
 
-template <int G, bool BF16>
-__device__ __forceinline__ void tuple_field_vec(uint32_t ent, int nhalf, uint32_t base,
-                                                uint64_t* acc)
+// FP32 operand: V / 2 packed pairs.
+template <int G, int V>
+__device__ __forceinline__ void tuple_field_f32(uint32_t ent, int nhalf, uint32_t base, float* acc)
 {
-    using GT = Gather<BF16>;
+    constexpr int SH = V == 4 ? 4 : 3;
+    uint64_t s[V / 2];
 #pragma unroll
-    for (int k = 0; k < GT::NP; ++k) acc[k] = 0ull;
+    for (int k = 0; k < V / 2; ++k) s[k] = 0ull;
     for (int hc = 0; hc < nhalf; hc += 2) {
         const uint4 e = lds128(ent + (uint32_t)(hc >> 1) * (G * 16u));
         const uint32_t ew[4] = {e.x, e.y, e.z, e.w};
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (h == 1 && hc + 1 >= nhalf) break;
-            GT a, b, c, d;
-            a.load(base + ((ew[2 * h] & 0xffffu) << 4));
-            b.load(base + ((ew[2 * h] >> 16) << 4));
-            c.load(base + ((ew[2 * h + 1] & 0xffffu) << 4));
-            d.load(base + ((ew[2 * h + 1] >> 16) << 4));
+            uint32_t v[4][V];
+            lds_words<V>(base + ((ew[2 * h] & 0xffffu) << SH), v[0]);
+            lds_words<V>(base + ((ew[2 * h] >> 16) << SH), v[1]);
+            lds_words<V>(base + ((ew[2 * h + 1] & 0xffffu) << SH), v[2]);
+            lds_words<V>(base + ((ew[2 * h + 1] >> 16) << SH), v[3]);
 #pragma unroll
-            for (int k = 0; k < GT::NP; ++k)
-                acc[k] = add2(acc[k], add2(add2(a.v[k], b.v[k]), add2(c.v[k], d.v[k])));
+            for (int k = 0; k < V / 2; ++k) {
+                const uint64_t a = pack2(v[0][2 * k], v[0][2 * k + 1]);
+                const uint64_t b = pack2(v[1][2 * k], v[1][2 * k + 1]);
+                const uint64_t c = pack2(v[2][2 * k], v[2][2 * k + 1]);
+                const uint64_t d = pack2(v[3][2 * k], v[3][2 * k + 1]);
+                s[k] = add2(s[k], add2(add2(a, b), add2(c, d)));
+            }
         }
     }
+#pragma unroll
+    for (int u = 0; u < V; ++u) acc[u] = (u & 1) ? hi_f(s[u >> 1]) : lo_f(s[u >> 1]);
+}
+
+template <int G, int V, bool BF16>
+__device__ __forceinline__ void tuple_field(uint32_t ent, int nhalf, uint32_t base, float* acc)
+{
+    if constexpr (BF16) tuple_field_bf16<G, V>(ent, nhalf, base, acc);
+    else tuple_field_f32<G, V>(ent, nhalf, base, acc);
+}
+
+// Both halves of the next operand buffer, +x at a and -x at an.
+template <int V, bool BF16>
+__device__ __forceinline__ void store_operand(uint32_t a, uint32_t an, const float* x)
+{
+    constexpr int NW = BF16 ? V / 2 : V;
+    uint32_t w[NW], n[NW];
+#pragma unroll
+    for (int k = 0; k < NW; ++k) {
+        if constexpr (BF16) {
+            const __nv_bfloat162 b2 = __floats2bfloat162_rn(x[2 * k], x[2 * k + 1]);
+            w[k] = *reinterpret_cast<const uint32_t*>(&b2);
+            n[k] = w[k] ^ 0x80008000u;
+        } else {
+            w[k] = __float_as_uint(x[k]);
+            n[k] = w[k] ^ 0x80000000u;
+        }
+    }
+    sts_words<NW>(a, w);
+    sts_words<NW>(an, n);
 }
 
 struct VArgs {
@@ -227,10 +319,10 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
     k_sparse_md_vec(const VArgs a)
 {
     constexpr int ES = BF16 ? 2 : 4;
-    constexpr int V = 16 / ES;     // replicas per lane
-    constexpr int LPR = RB / V;    // lanes per row
-    constexpr int G = 32 / LPR;    // rows per warp instruction
-    constexpr int NP = V / 2;
+    constexpr int V = vec_of(RB, BF16);   // replicas per lane
+    constexpr int LPR = RB / V;           // lanes per row
+    constexpr int G = 32 / LPR;           // rows per warp instruction
+    constexpr uint32_t VB = V * ES;       // bytes of a gather
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
     const uint32_t half_bytes = (uint32_t)a.Npad * RB * ES;
@@ -315,18 +407,13 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
                 }
             }
 #pragma unroll
-            for (int k4 = 0; k4 < V / 4; ++k4) {
-                uint4 x = make_uint4(0, 0, 0, 0), y = make_uint4(0, 0, 0, 0);
-                if (rok[kk]) {
-                    x = lds128((BF16 ? master : op0) + (re0[kk] + 4 * k4) * 4u);
-                    y = lds128(ps + (re0[kk] + 4 * k4) * 4u);
-                    // from here to the end of the run ps holds the window sums
-                    sts128(ps + (re0[kk] + 4 * k4) * 4u, make_uint4(0, 0, 0, 0));
-                }
-                rphi[kk][4 * k4] = __uint_as_float(x.x); rphi[kk][4 * k4 + 1] = __uint_as_float(x.y);
-                rphi[kk][4 * k4 + 2] = __uint_as_float(x.z); rphi[kk][4 * k4 + 3] = __uint_as_float(x.w);
-                rp[kk][4 * k4] = __uint_as_float(y.x); rp[kk][4 * k4 + 1] = __uint_as_float(y.y);
-                rp[kk][4 * k4 + 2] = __uint_as_float(y.z); rp[kk][4 * k4 + 3] = __uint_as_float(y.w);
+            for (int u = 0; u < V; ++u) rphi[kk][u] = rp[kk][u] = 0.f;
+            if (rok[kk]) {
+                const float zero[V] = {};
+                lds_state<V>((BF16 ? master : op0) + re0[kk] * 4u, rphi[kk]);
+                lds_state<V>(ps + re0[kk] * 4u, rp[kk]);
+                // from here to the end of the run ps holds the window sums
+                sts_state<V>(ps + re0[kk] * 4u, zero);
             }
         }
         const int nk = wend - wbeg;
@@ -339,14 +426,7 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
             for (int kk = 0; kk < RS; ++kk) {
                 if (kk >= nk) break;
                 float Lsum[V];
-                if constexpr (BF16) {
-                    tuple_field_bf16<G>(rent[kk], rnh[kk], cur + (uint32_t)q * 16u, Lsum);
-                } else {
-                    uint64_t acc[NP];
-                    tuple_field_vec<G, BF16>(rent[kk], rnh[kk], cur + (uint32_t)q * 16u, acc);
-#pragma unroll
-                    for (int u = 0; u < V; ++u) Lsum[u] = (u & 1) ? hi_f(acc[u >> 1]) : lo_f(acc[u >> 1]);
-                }
+                tuple_field<G, V, BF16>(rent[kk], rnh[kk], cur + (uint32_t)q * VB, Lsum);
                 if (!rok[kk]) continue;
 #pragma unroll
                 for (int u = 0; u < V; ++u) {
@@ -356,35 +436,13 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
                     rp[kk][u] = rp[kk][u] - fmaf(cf.x, pw, cf.y * L);
                     rphi[kk][u] = fmaf(cf.z, rp[kk][u], rphi[kk][u]);
                 }
-                if constexpr (BF16) {
-                    uint32_t pk[4];
-#pragma unroll
-                    for (int k2 = 0; k2 < 4; ++k2) {
-                        __nv_bfloat162 b2 = __floats2bfloat162_rn(rphi[kk][2 * k2], rphi[kk][2 * k2 + 1]);
-                        pk[k2] = *reinterpret_cast<uint32_t*>(&b2);
-                    }
-                    sts128(nxt + re0[kk] * 2u, make_uint4(pk[0], pk[1], pk[2], pk[3]));
-                    sts128(nxt + half_bytes + re0[kk] * 2u,
-                           make_uint4(pk[0] ^ 0x80008000u, pk[1] ^ 0x80008000u, pk[2] ^ 0x80008000u,
-                                      pk[3] ^ 0x80008000u));
-                } else {
-                    const uint4 f = make_uint4(__float_as_uint(rphi[kk][0]), __float_as_uint(rphi[kk][1]),
-                                               __float_as_uint(rphi[kk][2]), __float_as_uint(rphi[kk][3]));
-                    sts128(nxt + re0[kk] * 4u, f);
-                    sts128(nxt + half_bytes + re0[kk] * 4u,
-                           make_uint4(f.x ^ 0x80000000u, f.y ^ 0x80000000u, f.z ^ 0x80000000u,
-                                      f.w ^ 0x80000000u));
-                }
+                store_operand<V, BF16>(nxt + re0[kk] * ES, nxt + half_bytes + re0[kk] * ES, rphi[kk]);
                 if (in_win) {
+                    float w[V];
+                    lds_state<V>(ps + re0[kk] * 4u, w);
 #pragma unroll
-                    for (int k4 = 0; k4 < V / 4; ++k4) {
-                        const uint32_t o = ps + (re0[kk] + 4 * k4) * 4u;
-                        const uint4 w = lds128(o);
-                        sts128(o, make_uint4(__float_as_uint(__uint_as_float(w.x) + rphi[kk][4 * k4]),
-                                             __float_as_uint(__uint_as_float(w.y) + rphi[kk][4 * k4 + 1]),
-                                             __float_as_uint(__uint_as_float(w.z) + rphi[kk][4 * k4 + 2]),
-                                             __float_as_uint(__uint_as_float(w.w) + rphi[kk][4 * k4 + 3])));
-                    }
+                    for (int u = 0; u < V; ++u) w[u] += rphi[kk][u];
+                    sts_state<V>(ps + re0[kk] * 4u, w);
                 }
             }
             __syncthreads();
@@ -395,18 +453,12 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
 #pragma unroll
         for (int kk = 0; kk < RS; ++kk) {
             if (!rok[kk]) continue;
-#pragma unroll
-            for (int k4 = 0; k4 < V / 4; ++k4) {
-                const uint32_t o = (re0[kk] + 4 * k4) * 4u;
-                sts128(dead + o, lds128(ps + o));
-                sts128(ps + o, make_uint4(__float_as_uint(rp[kk][4 * k4]), __float_as_uint(rp[kk][4 * k4 + 1]),
-                                          __float_as_uint(rp[kk][4 * k4 + 2]),
-                                          __float_as_uint(rp[kk][4 * k4 + 3])));
-                sts128((BF16 ? master : fin) + o,
-                       make_uint4(__float_as_uint(rphi[kk][4 * k4]), __float_as_uint(rphi[kk][4 * k4 + 1]),
-                                  __float_as_uint(rphi[kk][4 * k4 + 2]),
-                                  __float_as_uint(rphi[kk][4 * k4 + 3])));
-            }
+            const uint32_t o = re0[kk] * 4u;
+            float w[V];
+            lds_state<V>(ps + o, w);
+            sts_state<V>(dead + o, w);
+            sts_state<V>(ps + o, rp[kk]);
+            sts_state<V>((BF16 ? master : fin) + o, rphi[kk]);
         }
         __syncthreads();
     } else
@@ -419,31 +471,15 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
             const int t = __ldg(a.tuple_list + k);
             const int4 tp = __ldg(a.tuples + t);
             float Lsum[V];
-            if constexpr (BF16) {
-                tuple_field_bf16<G>(s0 + ((uint32_t)tp.x * G + g) * 16u, tp.y,
-                                    cur + (uint32_t)q * 16u, Lsum);
-            } else {
-                uint64_t acc[NP];
-                tuple_field_vec<G, BF16>(s0 + ((uint32_t)tp.x * G + g) * 16u, tp.y,
-                                         cur + (uint32_t)q * 16u, acc);
-#pragma unroll
-                for (int u = 0; u < V; ++u) Lsum[u] = (u & 1) ? hi_f(acc[u >> 1]) : lo_f(acc[u >> 1]);
-            }
+            tuple_field<G, V, BF16>(s0 + ((uint32_t)tp.x * G + g) * 16u, tp.y,
+                                    cur + (uint32_t)q * VB, Lsum);
             const int row = __ldg(a.tuple_rows + t * G + g);
             if (row < 0) continue;
             const uint32_t e0 = (uint32_t)(__ldg(a.slot_of_row + row) * RB + q * V);
             const float hr = a.h ? 2.f * __ldg(a.h + row) : 0.f;
-            // this lane's V replicas of `row`, 16-byte vectors
             float phi[V], p[V];
-#pragma unroll
-            for (int k4 = 0; k4 < V / 4; ++k4) {
-                const uint4 x = lds128((BF16 ? master : cur) + (e0 + 4 * k4) * 4u);
-                const uint4 y = lds128(ps + (e0 + 4 * k4) * 4u);
-                phi[4 * k4] = __uint_as_float(x.x); phi[4 * k4 + 1] = __uint_as_float(x.y);
-                phi[4 * k4 + 2] = __uint_as_float(x.z); phi[4 * k4 + 3] = __uint_as_float(x.w);
-                p[4 * k4] = __uint_as_float(y.x); p[4 * k4 + 1] = __uint_as_float(y.y);
-                p[4 * k4 + 2] = __uint_as_float(y.z); p[4 * k4 + 3] = __uint_as_float(y.w);
-            }
+            lds_state<V>((BF16 ? master : cur) + e0 * 4u, phi);
+            lds_state<V>(ps + e0 * 4u, p);
 #pragma unroll
             for (int u = 0; u < V; ++u) {
                 const float L = Lsum[u] + hr * fabsf(phi[u]);
@@ -452,40 +488,18 @@ __global__ void __launch_bounds__(REG > 0 ? reg_threads(REG, BF16) : kMaxThreads
                 p[u] = p[u] - fmaf(cf.x, pw, cf.y * L);
                 phi[u] = fmaf(cf.z, p[u], phi[u]);
             }
+            sts_state<V>(ps + e0 * 4u, p);
+            if constexpr (BF16) sts_state<V>(master + e0 * 4u, phi);
+            store_operand<V, BF16>(nxt + e0 * ES, nxt + half_bytes + e0 * ES, phi);
+            if (in_win) {
 #pragma unroll
-            for (int k4 = 0; k4 < V / 4; ++k4) {
-                const uint32_t o = (e0 + 4 * k4) * 4u;
-                sts128(ps + o, make_uint4(__float_as_uint(p[4 * k4]), __float_as_uint(p[4 * k4 + 1]),
-                                          __float_as_uint(p[4 * k4 + 2]), __float_as_uint(p[4 * k4 + 3])));
-                const uint4 f = make_uint4(__float_as_uint(phi[4 * k4]), __float_as_uint(phi[4 * k4 + 1]),
-                                           __float_as_uint(phi[4 * k4 + 2]), __float_as_uint(phi[4 * k4 + 3]));
-                if constexpr (BF16) {
-                    sts128(master + o, f);
-                } else {
-                    sts128(nxt + o, f);
-                    sts128(nxt + half_bytes + o, make_uint4(f.x ^ 0x80000000u, f.y ^ 0x80000000u,
-                                                            f.z ^ 0x80000000u, f.w ^ 0x80000000u));
-                }
-                if (in_win) {
-                    float4* wp = reinterpret_cast<float4*>(gw + e0 + 4 * k4);
+                for (int k = 0; k < V; k += 4) {   // V >= 4 without register state
+                    float4* wp = reinterpret_cast<float4*>(gw + e0 + k);
                     float4 w = *wp;
-                    w.x += phi[4 * k4]; w.y += phi[4 * k4 + 1];
-                    w.z += phi[4 * k4 + 2]; w.w += phi[4 * k4 + 3];
+                    w.x += phi[k]; w.y += phi[k + 1];
+                    w.z += phi[k + 2]; w.w += phi[k + 3];
                     *wp = w;
                 }
-            }
-            if constexpr (BF16) {
-                // 8 BF16 values (16 bytes) into both halves of the next operand buffer
-                uint32_t pk[4];
-#pragma unroll
-                for (int k2 = 0; k2 < 4; ++k2) {
-                    __nv_bfloat162 b2 = __floats2bfloat162_rn(phi[2 * k2], phi[2 * k2 + 1]);
-                    pk[k2] = *reinterpret_cast<uint32_t*>(&b2);
-                }
-                sts128(nxt + e0 * 2u, make_uint4(pk[0], pk[1], pk[2], pk[3]));
-                sts128(nxt + half_bytes + e0 * 2u,
-                       make_uint4(pk[0] ^ 0x80008000u, pk[1] ^ 0x80008000u, pk[2] ^ 0x80008000u,
-                                  pk[3] ^ 0x80008000u));
             }
         }
         __syncthreads();
@@ -520,10 +534,10 @@ template <int RB, bool BF16>
 __global__ void __launch_bounds__(kMaxThreads, 1) k_sparse_field_vec(const VArgs a)
 {
     constexpr int ES = BF16 ? 2 : 4;
-    constexpr int V = 16 / ES;
+    constexpr int V = vec_of(RB, BF16);
     constexpr int LPR = RB / V;
     constexpr int G = 32 / LPR;
-    constexpr int NP = V / 2;
+    constexpr uint32_t VB = V * ES;
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
     const uint32_t half_bytes = (uint32_t)a.Npad * RB * ES;
@@ -554,16 +568,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sparse_field_vec(const VArgs
         const int t = __ldg(a.tuple_list + k);
         const int4 tp = __ldg(a.tuples + t);
         float Lsum[V];
-        if constexpr (BF16) {
-            tuple_field_bf16<G>(s0 + ((uint32_t)tp.x * G + g) * 16u, tp.y, op0 + (uint32_t)q * 16u,
-                                Lsum);
-        } else {
-            uint64_t acc[NP];
-            tuple_field_vec<G, BF16>(s0 + ((uint32_t)tp.x * G + g) * 16u, tp.y,
-                                     op0 + (uint32_t)q * 16u, acc);
-#pragma unroll
-            for (int u = 0; u < V; ++u) Lsum[u] = (u & 1) ? hi_f(acc[u >> 1]) : lo_f(acc[u >> 1]);
-        }
+        tuple_field<G, V, BF16>(s0 + ((uint32_t)tp.x * G + g) * 16u, tp.y, op0 + (uint32_t)q * VB, Lsum);
         const int row = __ldg(a.tuple_rows + t * G + g);
         if (row < 0) continue;
 #pragma unroll
@@ -577,7 +582,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sparse_field_vec(const VArgs
     }
 }
 
-int vec_width(int prec) { return prec == HQA_PREC_BF16 ? 8 : 4; }
+// Rows per bank phase: as many as 128 bytes hold.
+int vec_phase(int RB, int prec) { return std::max(1, 128 / (RB * (prec == HQA_PREC_BF16 ? 2 : 4))); }
 
 // ---------------------------------------------------------------------------
 // host: plan construction
@@ -705,19 +711,19 @@ void colour_phase(const std::vector<std::vector<PhaseEntry>>& lists, int P, int 
 bool hqa_vec_supported(const hqa_ctx* ctx, int RB, int prec)
 {
     if (!ctx->unit) return false;
-    const int V = vec_width(prec);
+    const int V = vec_of(RB, prec == HQA_PREC_BF16);
     if (RB < V || RB > 32) return false;
-    const int es = prec == HQA_PREC_BF16 ? 2 : 4;
-    const int P = std::max(1, 128 / (RB * es));
+    // 8-byte gathers only with the state in registers (at most 64 tuples of 32 rows)
+    if (V < (prec == HQA_PREC_BF16 ? 8 : 4) && ctx->N > 2048) return false;
+    const int P = vec_phase(RB, prec);
     const int64_t Npad = ((int64_t)ctx->N + P - 1) / P * P + P;
-    // u16 offsets in units of 16 bytes over both halves of a step buffer
-    return 2 * Npad * RB * es / 16 < 65536;
+    // u16 offsets in units of one gather over both halves of a step buffer
+    return 2 * Npad * RB / V < 65536;
 }
 
 static int64_t vec_npad(const hqa_ctx* ctx, int RB, int prec)
 {
-    const int es = prec == HQA_PREC_BF16 ? 2 : 4;
-    const int P = std::max(1, 128 / (RB * es));
+    const int P = vec_phase(RB, prec);
     return ((int64_t)ctx->N + P - 1) / P * P + P;
 }
 
@@ -742,14 +748,13 @@ hqa_status hqa_vec_plan(hqa_ctx* ctx, int RB, int prec, const SparsePlan** out)
     }
     // building a plan allocates and uploads: not possible inside a capture
     if (hqa_capturing()) return hqa_capture_note(HQA_ERR_UNSUPPORTED);
-    const int es = prec == HQA_PREC_BF16 ? 2 : 4;
-    const int V = vec_width(prec);
+    const int V = vec_of(RB, prec == HQA_PREC_BF16);
     const int LPR = RB / V;
     const int G = 32 / LPR;
-    const int P = std::max(1, 128 / (RB * es));   // rows per 8-lane phase
+    const int P = vec_phase(RB, prec);            // rows per 8-lane (16-lane) phase
     const int N = ctx->N;
     const int Npad = (int)vec_npad(ctx, RB, prec);
-    const int unit = RB * es / 16;                // one slot in 16-byte units
+    const int unit = LPR;                         // one slot in gathers
     // all neighbours of each row with their sign
     std::vector<std::vector<std::pair<int, bool>>> nb(N);
     for (int i = 0; i < N; ++i)
@@ -795,6 +800,7 @@ hqa_status hqa_vec_plan(hqa_ctx* ctx, int RB, int prec, const SparsePlan** out)
         HostRng rng{0x5EEDull + (uint64_t)N * 131 + (uint64_t)RB};
         const int64_t iters = (int64_t)40 * N;
         std::vector<int> touched;
+        for (auto& o : occ) std::sort(o.begin(), o.end());   // once, so that two merge
         for (int64_t itn = 0; itn < iters; ++itn) {
             const auto& pr = phase_rows[rng.next() % (uint64_t)nphases];
             if (pr.size() < 2) continue;
@@ -802,10 +808,8 @@ hqa_status hqa_vec_plan(hqa_ctx* ctx, int RB, int prec, const SparsePlan** out)
             int b = pr[rng.next() % pr.size()];
             if (a == b) continue;
             const int qa = grp[a], qb = grp[b];
-            touched.clear();
-            for (int ti : occ[a]) touched.push_back(ti);
-            for (int ti : occ[b]) touched.push_back(ti);
-            std::sort(touched.begin(), touched.end());
+            touched.resize(occ[a].size() + occ[b].size());
+            std::merge(occ[a].begin(), occ[a].end(), occ[b].begin(), occ[b].end(), touched.begin());
             touched.erase(std::unique(touched.begin(), touched.end()), touched.end());
             int before = 0;
             for (int ti : touched) before += term_cost(ti);
@@ -992,10 +996,13 @@ static cudaError_t launch_vec_md(const VArgs& a, int threads, size_t smem, cudaS
         else k_sparse_md_vec<RB, BF16, 4><<<blocks, threads, smem, st>>>(a);
         return cudaGetLastError();
     }
-    cudaError_t e = hqa_smem_attr((const void*)k_sparse_md_vec<RB, BF16, 0>, smem);
-    if (e != cudaSuccess) return e;
-    k_sparse_md_vec<RB, BF16, 0><<<(a.R + RB - 1) / RB, threads, smem, st>>>(a);
-    return cudaGetLastError();
+    if constexpr (vec_of(RB, BF16) >= 4 && RB >= (BF16 ? 8 : 4)) {
+        cudaError_t e = hqa_smem_attr((const void*)k_sparse_md_vec<RB, BF16, 0>, smem);
+        if (e != cudaSuccess) return e;
+        k_sparse_md_vec<RB, BF16, 0><<<(a.R + RB - 1) / RB, threads, smem, st>>>(a);
+        return cudaGetLastError();
+    }
+    return cudaErrorInvalidValue;   // 8-byte gathers: always with state in registers
 }
 
 template <int RB, bool BF16>
@@ -1020,8 +1027,9 @@ static cudaError_t dispatch_vec(bool field, int RB, bool bf, const VArgs& a, int
     HQA_VEC_CASE(32)
     HQA_VEC_CASE(16)
     HQA_VEC_CASE(8)
-    if (RB == 4 && !bf) return field ? launch_vec_field<4, false>(a, threads, smem, st)
-                                     : launch_vec_md<4, false>(a, threads, smem, st);
+    HQA_VEC_CASE(4)
+    if (RB == 2 && !bf) return field ? launch_vec_field<2, false>(a, threads, smem, st)
+                                     : launch_vec_md<2, false>(a, threads, smem, st);
 #undef HQA_VEC_CASE
     return cudaErrorInvalidValue;
 }
