@@ -742,6 +742,11 @@ static hqa_status run_impl(hqa_ctx* ctx, const hqa_schedule* sched, double dt, i
     else if (plan->vec)
         s = hqa_vec_launch_md(ctx, plan, ctx->d_sched, steps, sched->window, replicas, seed, o.init,
                               o.phi0, o.p0, sched->M, out->phi, out->p, phibar, st);
+    else if (o.kernel == HQA_KERNEL_AUTO && o.replicas_per_block == 0 && plan->RB == 1 &&
+             hqa_complete_possible(ctx, replicas))
+        s = hqa_complete_launch_md(ctx, o.precision, ctx->d_sched, steps, sched->window, replicas,
+                                   seed, o.init, o.phi0, o.p0, sched->M, out->phi, out->p, phibar,
+                                   st);
     else
         s = hqa_sparse_launch_md(ctx, plan, ctx->d_sched, steps, sched->window, replicas, seed,
                                  o.init, o.phi0, o.p0, sched->M, out->phi, out->p, phibar, st);
