@@ -321,6 +321,8 @@ def kernel_name(hqa, plan, prec_name):
         return f"k_dense_md<{plan['replicas_per_block'] // 2},*,{kseg},*,*,{f16},*,*,*>"
     if k == hqa.KERNEL_STREAM:
         return f"k_sparse_stream<{'true' if prec_name == 'PREC_BF16' else 'false'}>"
+    if k == hqa.KERNEL_SCALAR and plan.get("balance") == 1.0:
+        return f"k_md_complete<*,{'true' if prec_name == 'PREC_BF16' else 'false'}>"
     base = "k_sparse_md_vec" if k == hqa.KERNEL_VECTOR else "k_sparse_md"
     return f"{base}<{plan['replicas_per_block']},{'true' if prec_name == 'PREC_BF16' else 'false'}>"
 
@@ -549,7 +551,10 @@ def measure(name, args, hqa, torch, timer, dev, ws, rank, headline):
                 "note": "persistent batch kernel and replica blocking picked by the autotuner"}
         base = {hqa.KERNEL_LOWDEG: "k_batch_lowdeg", hqa.KERNEL_SCALAR: "k_sparse_md_batch"}.get(
             kb, "k_batch_lowdeg|k_sparse_md_batch")
-        kname = f"{base}<{rb or '*'},{'true' if hv['prec_name'] == 'PREC_BF16' else 'false'}>"
+        bf = "true" if hv["prec_name"] == "PREC_BF16" else "false"
+        # members of at most 5000 spins without fields: the register form from two replicas on
+        kname = (f"k_batch_lowdeg_reg<{bf}>" if kb == hqa.KERNEL_LOWDEG and rb >= 2
+                 else f"{base}<{rb or '*'},{bf}>")
     else:
         plan = ctx.plan(R, precision=hv["prec"], kernel=hv["kernel"])
         kname = kernel_name(hqa, plan, hv["prec_name"])
@@ -560,18 +565,20 @@ def measure(name, args, hqa, torch, timer, dev, ws, rank, headline):
         kseg = 1
         if hv["prec_name"].endswith("X2"):
             kseg = 3 if real else 2
+        elif kname == "k_dense_f32":
+            kseg = 6 if real else 3     # products of BF16 slices per FP32 product
         flops = 2.0 * N * N * R * S / chunks            # algorithmic per launch: the field GEMM
         t_launch = t_run / chunks
         achieved = flops / t_launch / 1e12
-        if hv["prec_name"] == "PREC_FP32":
+        if hv["prec_name"] == "PREC_FP32" and kname != "k_dense_f32":
             sm = torch.cuda.get_device_properties(dev).multi_processor_count
             peak = sm * 128 * 2 * 2070e6 / 1e12           # FP32 FMA lanes x 2 flop x max clock
             roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak,
                     "peak_source": "derived: SMs x 128 FP32 lanes x 2 flop x 2070 MHz"}
         else:
-            # the kernel is timed on its own: the burst peak; a split operand issues
-            # kseg MMA passes for each algorithmic flop
+            # the kernel is timed on its own: the burst peak; a split or sliced operand
+            # issues kseg MMA passes for each algorithmic flop
             roof = {"bound": "tensor", "achieved": achieved, "peak": pk["bf16_burst"],
                     "unit": "TFLOP/s", "frac": achieved / pk["bf16_burst"],
                     "issued_tflops": achieved * kseg,

@@ -739,14 +739,14 @@ static hqa_status run_impl(hqa_ctx* ctx, const hqa_schedule* sched, double dt, i
         s = hqa_stream_launch_md(ctx, o.precision, ctx->d_sched, steps, sched->window, replicas,
                                  seed, o.init, o.phi0, o.p0, sched->M, out->phi, out->p, phibar,
                                  st);
-    else if (plan->vec)
-        s = hqa_vec_launch_md(ctx, plan, ctx->d_sched, steps, sched->window, replicas, seed, o.init,
-                              o.phi0, o.p0, sched->M, out->phi, out->p, phibar, st);
-    else if (o.kernel == HQA_KERNEL_AUTO && o.replicas_per_block == 0 && plan->RB == 1 &&
+    else if (o.kernel == HQA_KERNEL_AUTO && o.replicas_per_block == 0 &&
              hqa_complete_possible(ctx, replicas))
         s = hqa_complete_launch_md(ctx, o.precision, ctx->d_sched, steps, sched->window, replicas,
                                    seed, o.init, o.phi0, o.p0, sched->M, out->phi, out->p, phibar,
                                    st);
+    else if (plan->vec)
+        s = hqa_vec_launch_md(ctx, plan, ctx->d_sched, steps, sched->window, replicas, seed, o.init,
+                              o.phi0, o.p0, sched->M, out->phi, out->p, phibar, st);
     else
         s = hqa_sparse_launch_md(ctx, plan, ctx->d_sched, steps, sched->window, replicas, seed,
                                  o.init, o.phi0, o.p0, sched->M, out->phi, out->p, phibar, st);
@@ -942,6 +942,17 @@ hqa_status hqa_plan_query(hqa_ctx* ctx, int32_t replicas, const hqa_run_opts* op
         out->smem_bytes = 0;
         out->chunks = 1;
         out->pad_ratio = (double)((replicas + V - 1) / V * V) / replicas;
+        out->conflict_ratio = 1.0;
+        out->balance = 1.0;
+        return HQA_OK;
+    }
+    if (o.kernel == HQA_KERNEL_AUTO && o.replicas_per_block == 0 && hqa_complete_possible(ctx, replicas)) {
+        out->kernel = HQA_KERNEL_SCALAR;
+        out->replicas_per_block = 1;
+        out->blocks = replicas;
+        hqa_complete_shape(ctx, &out->threads, &out->smem_bytes);
+        out->chunks = 1;
+        out->pad_ratio = 1.0;
         out->conflict_ratio = 1.0;
         out->balance = 1.0;
         return HQA_OK;

@@ -275,6 +275,7 @@ hqa_status hqa_batch_launch_md(hqa_ctx* batch, int RB, int prec, const StepCoef*
 int hqa_sparse_pick_rb(const hqa_ctx* ctx, int32_t R, int prec);
 // sparse_complete.cu: few replicas of a small complete graph
 bool hqa_complete_possible(const hqa_ctx* ctx, int32_t R);
+void hqa_complete_shape(const hqa_ctx* ctx, int32_t* threads, int64_t* smem_bytes);
 hqa_status hqa_complete_launch_md(hqa_ctx* ctx, int prec, const StepCoef* d_sched, int64_t S,
                                   int32_t W, int32_t R, uint64_t seed, int init, const float* phi0,
                                   const float* p0, int M, float* phi_out, float* p_out,
