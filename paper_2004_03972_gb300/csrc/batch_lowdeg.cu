@@ -41,7 +41,7 @@ __host__ __device__ constexpr uint32_t ld_item_bytes(int N, int RB, bool bf16, b
 
 // Register-resident form: units (a spin and 2 replicas at RB = 2, 4 above) per
 // thread that its registers hold without spilling, and the shared memory of its
-// operand (two step buffers, each row and its negative).
+// operand (two step buffers).
 __host__ __device__ constexpr int ld_reg_units(int N, int RB)
 {
     return (N * (RB >= 8 ? RB / 4 : 1) + kLdThreads - 1) / kLdThreads;
@@ -56,10 +56,10 @@ __host__ __device__ constexpr bool ld_win_in_regs(int RB, int K)
 {
     return K * (RB >= 4 ? 4 : 2) <= 6;
 }
-__host__ __device__ constexpr uint32_t ld_reg_bytes(int N, int RB, bool bf16)
+__host__ __device__ constexpr uint32_t ld_reg_bytes(int N, int RB)
 {
     const int K = ld_reg_units(N, RB);
-    return align16(4u * (uint32_t)(N + 1) * RB * (bf16 ? 2u : 4u)) +
+    return align16(8u * (uint32_t)(N + 1) * RB) +   // FP32 rows, or BF16 rows of both signs
            (ld_win_in_regs(RB, K) ? 0u : (uint32_t)K * kLdThreads * (RB >= 4 ? 16u : 8u));
 }
 __host__ __device__ constexpr int ld_code(int RB, int K) { return RB * 16 + K; }
@@ -365,43 +365,40 @@ __global__ void __launch_bounds__(kLdThreads, 1) k_batch_lowdeg(const LdArgs a)
 // ---- state in registers -------------------------------------------------------
 // A thread owns the same K units (a spin, PR replicas) of its item at every step,
 // so momentum, window sums, flux and list stay in its registers; shared memory
-// holds the operand alone, with a negated copy of every row ([+ N + 1 rows |
-// - N + 1 rows], two step buffers), so that a list entry is a row number and a
-// gather needs no sign.  k_batch_lowdeg was bound by instructions: per spin and
-// pair about 110, of which the kick needs ten; shared-memory wavefronts came
-// next, a third of them list, momentum and window sums.  96 members of N = 200
-// to 5000 x 64 replicas, 100 steps in FP32, all in the window: 3157 -> 2484 us,
-// the same bits.
+// holds the operand alone.  k_batch_lowdeg was bound by instructions: per spin and
+// pair about 110, of which the kick needs ten; shared-memory wavefronts came next, a
+// third of them list, momentum and window sums.  What bounds this form is the
+// wavefronts of the gathers (91 % of the shared pipe busy, issue 30 %), so an FP32
+// row is stored once and its sign applied on arrival; both signs stored took
+// 2486 us.  BF16 rows, half as wide, are stored with both signs: the sign
+// arithmetic on their halves spilled.  96 members of N = 200 to 5000 x 64 replicas,
+// 100 steps in FP32, all in the window: 3157 -> 2072 us, the same bits.
 
 template <bool BF16, int PR>
 struct LdVec;                                   // PR replicas of one operand row
-template <> struct LdVec<false, 2> {
-    static __device__ __forceinline__ void load(uint32_t a, uint64_t* v)
+template <int PR> struct LdVec<false, PR> {
+    // v = +-row: the sign bits of sg (0 or 0x80000000) flip both halves of a pair
+    static __device__ __forceinline__ void load(uint32_t a, uint32_t sg, uint64_t* v)
     {
-        const uint2 x = lds64(a);
-        v[0] = (uint64_t)x.x | ((uint64_t)x.y << 32);
+        const uint64_t s2 = (uint64_t)sg | ((uint64_t)sg << 32);
+        if constexpr (PR == 2) {
+            const uint2 x = lds64(a);
+            v[0] = ((uint64_t)x.x | ((uint64_t)x.y << 32)) ^ s2;
+        } else {
+            uint64_t x, y;
+            asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "r"(a));
+            v[0] = x ^ s2;
+            v[PR / 2 - 1] = y ^ s2;
+        }
     }
-    static __device__ __forceinline__ void store(uint32_t a, uint32_t an, const uint64_t* v)
+    static __device__ __forceinline__ void store(uint32_t a, uint32_t, const uint64_t* v)
     {
-        const uint2 x = make_uint2((uint32_t)v[0], (uint32_t)(v[0] >> 32));
-        sts64(a, x);
-        sts64(an, make_uint2(x.x ^ 0x80000000u, x.y ^ 0x80000000u));
-    }
-};
-template <> struct LdVec<false, 4> {
-    static __device__ __forceinline__ void load(uint32_t a, uint64_t* v)
-    {
-        asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(a));
-    }
-    static __device__ __forceinline__ void store(uint32_t a, uint32_t an, const uint64_t* v)
-    {
-        constexpr uint64_t sg = 0x8000000080000000ull;
-        asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(a), "l"(v[0]), "l"(v[1]));
-        asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(an), "l"(v[0] ^ sg), "l"(v[1] ^ sg));
+        if constexpr (PR == 2) sts64(a, make_uint2((uint32_t)v[0], (uint32_t)(v[0] >> 32)));
+        else asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(a), "l"(v[0]), "l"(v[PR / 2 - 1]));
     }
 };
 template <int PR> struct LdVec<true, PR> {
-    static __device__ __forceinline__ void load(uint32_t a, uint64_t* v)
+    static __device__ __forceinline__ void load(uint32_t a, uint32_t, uint64_t* v)
     {
         uint32_t x[PR / 2];
         if constexpr (PR == 2) {
@@ -442,13 +439,15 @@ __device__ __forceinline__ void ld_item(const LdArgs& a, const LdMember& m, int 
     constexpr int PR = RB >= 4 ? 4 : 2, TR = RB / PR, NP = PR / 2;
     using V = LdVec<BF16, PR>;
     const int t = threadIdx.x, N = m.N, U = N * TR;
-    const uint32_t half = (uint32_t)(N + 1) * ROW, buf = 2u * half;
+    // NEG: a negated copy of the rows behind them, and list entries that name its rows
+    constexpr bool NEG = BF16;
+    const uint32_t half = (uint32_t)(N + 1) * ROW, buf = NEG ? 2u * half : half;
     const int row0 = t / TR, r0 = (t % TR) * PR;      // unit k: row0 + k * RSTEP, r0
     constexpr int RSTEP = kLdThreads / TR;
     const uint32_t lane = (uint32_t)r0 * (BF16 ? 2u : 4u);
     const uint32_t own = lane + (uint32_t)row0 * ROW;
 
-    // row N of the + halves is the lists' padding: zero in both step buffers
+    // row N is the lists' padding: zero in both step buffers
     if (t < 2 * (int)(ROW / 4u))
         sts32(s0 + (t & 1) * buf + (uint32_t)N * ROW + (uint32_t)(t >> 1) * 4u, 0.f);
     uint2 li[K];
@@ -467,14 +466,12 @@ __device__ __forceinline__ void ld_item(const LdArgs& a, const LdMember& m, int 
         }
         const int row = row0 + k * RSTEP;
         if (t + k * kLdThreads >= U) continue;
-        const uint2 l = __ldg(m.lists + row);
-        const uint32_t neg = (uint32_t)(N + 1);
-        // bit 15 set -> the row of the negated half
-        const uint32_t e0 = (l.x & 0x7fffu) + ((l.x & 0x8000u) ? neg : 0u);
-        const uint32_t e1 = ((l.x >> 16) & 0x7fffu) + ((l.x >> 31) ? neg : 0u);
-        const uint32_t e2 = (l.y & 0x7fffu) + ((l.y & 0x8000u) ? neg : 0u);
-        const uint32_t e3 = ((l.y >> 16) & 0x7fffu) + ((l.y >> 31) ? neg : 0u);
-        li[k] = make_uint2(e0 | (e1 << 16), e2 | (e3 << 16));
+        li[k] = __ldg(m.lists + row);
+        if constexpr (NEG) {
+            const auto flat = [N](uint32_t e) { return (e & 0x7fffu) + ((e & 0x8000u) ? (uint32_t)(N + 1) : 0u); };
+            li[k] = make_uint2(flat(li[k].x & 0xffffu) | (flat(li[k].x >> 16) << 16),
+                               flat(li[k].y & 0xffffu) | (flat(li[k].y >> 16) << 16));
+        }
         float x[PR], q[PR];
 #pragma unroll
         for (int i = 0; i < PR; ++i) {
@@ -513,11 +510,12 @@ __device__ __forceinline__ void ld_item(const LdArgs& a, const LdMember& m, int 
         for (int k = 0; k < K; ++k) {
             if (k == K - 1 && t + k * kLdThreads >= U) continue;
             uint64_t v0[NP], v1[NP], v2[NP], v3[NP];
-            V::load(cur + lane + (li[k].x & 0xffffu) * ROW, v0);
-            V::load(cur + lane + (li[k].x >> 16) * ROW, v1);
-            V::load(cur + lane + (li[k].y & 0xffffu) * ROW, v2);
-            V::load(cur + lane + (li[k].y >> 16) * ROW, v3);
-            if constexpr (!FREG) V::load(cur + own + (uint32_t)(k * RSTEP) * ROW, f[k]);
+            constexpr uint32_t sign = 0x80000000u, mask = NEG ? 0xffffu : 0x7fffu;
+            V::load(cur + lane + (li[k].x & mask) * ROW, (li[k].x << 16) & sign, v0);
+            V::load(cur + lane + ((li[k].x >> 16) & mask) * ROW, li[k].x & sign, v1);
+            V::load(cur + lane + (li[k].y & mask) * ROW, (li[k].y << 16) & sign, v2);
+            V::load(cur + lane + ((li[k].y >> 16) & mask) * ROW, li[k].y & sign, v3);
+            if constexpr (!FREG) V::load(cur + own + (uint32_t)(k * RSTEP) * ROW, 0u, f[k]);
 #pragma unroll
             for (int c = 0; c < NP; ++c) {
                 const uint64_t L = add2(add2(v0[c], v1[c]), add2(v2[c], v3[c]));
@@ -554,7 +552,7 @@ __device__ __forceinline__ void ld_item(const LdArgs& a, const LdMember& m, int 
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         if (t + k * kLdThreads >= U) continue;
-        if constexpr (!FREG) V::load(cur + own + (uint32_t)(k * RSTEP) * ROW, f[k]);
+        if constexpr (!FREG) V::load(cur + own + (uint32_t)(k * RSTEP) * ROW, 0u, f[k]);
 #pragma unroll
         for (int i = 0; i < PR; ++i) {
             const int rep = rep0 + r0 + i;
@@ -722,7 +720,7 @@ hqa_status hqa_lowdeg_launch_md(hqa_ctx* b, int RB, int prec, const StepCoef* d_
     if (reg) {
         size_t need = 0;
         for (int k = 0; k < count; ++k)
-            need = std::max<size_t>(need, ld_reg_bytes(b->members[k]->N, raise ? mrb[k] : RB, bf));
+            need = std::max<size_t>(need, ld_reg_bytes(b->members[k]->N, raise ? mrb[k] : RB));
         reg = need <= b->smem_optin - 1024;
         if (reg) smem = need;
     }
