@@ -26,9 +26,9 @@
 // per SM); the rest stay in global memory.  That takes 68 of the 174 MB that a
 // step moved through L2 at N = 20000 x 256 in BF16, and one CTA per SM makes a
 // barrier 152 arrivals instead of one per 256 threads.  Per step there: BF16
-// 20.9 -> 14.7 us, FP32 20.6 -> 19.4 us (its gathers, 164 MB, then move at 10
-// TB/s); N = 8000 x 40 FP32 5.4 -> 4.1 us, mostly the barrier and two rounds of
-// gathers.
+// 20.9 -> 14.7 us, FP32 20.6 -> 19.4 us, and with the ranges cut at whole warps
+// (first_cell) 12.2 and 16.0; N = 8000 x 40 FP32 5.4 -> 4.1 us, mostly the barrier
+// and two rounds of gathers.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -263,6 +263,16 @@ __device__ __forceinline__ void get4(float* x, const float4* src)
     x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
 }
 
+// First cell of CTA b of g, in units of 32 where rows are a multiple of 32 vectors:
+// a warp then stays within one row (one list length, four full lines per gather).
+// N = 20000 x 256 BF16, 100 steps, 1888 -> 1637 us, FP32, 60 steps, 1454 -> 1250 us;
+// other row lengths, where a warp spans rows all the same, lost up to 9 %.
+__host__ __device__ inline int64_t cell_unit(int nv) { return nv % 32 == 0 ? 32 : 1; }
+__host__ __device__ inline int64_t first_cell(int64_t cells, int nv, int64_t b, int64_t g)
+{
+    return cells / cell_unit(nv) * b / g * cell_unit(nv);
+}
+
 // 16-byte state vectors of a cell: p, and in BF16 the FP32 master before it.
 template <bool BF16>
 constexpr int kPlanes = BF16 ? 4 : 1;
@@ -274,7 +284,7 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
     extern __shared__ float4 st[];   // [NP][nres], then (STAGED) the lists
     const int nv = a.Rpad / V;
     const int64_t cells = (int64_t)a.N * nv;
-    const int64_t c0 = cells * blockIdx.x / gridDim.x, c1 = cells * (blockIdx.x + 1) / gridDim.x;
+    const int64_t c0 = first_cell(cells, nv, blockIdx.x, gridDim.x), c1 = first_cell(cells, nv, blockIdx.x + 1, gridDim.x);
     const int mine = (int)(c1 - c0), nres = min(mine, a.nres);
     const int64_t first = c0 + threadIdx.x;
     const int i0 = (int)(first / nv), v0 = (int)(first % nv);
@@ -584,12 +594,14 @@ hqa_status hqa_stream_launch_md(hqa_ctx* ctx, int prec, const StepCoef* d_sched,
     const int nv = a.Rpad / (bf16 ? 8 : 4);
     size_t lists = 0;
     for (int b = 0; b < grid; ++b) {
-        const int64_t i0 = cells * b / grid / nv, i1 = (cells * (b + 1) / grid - 1) / nv;
+        const int64_t i0 = first_cell(cells, nv, b, grid) / nv;
+        const int64_t i1 = (first_cell(cells, nv, b + 1, grid) - 1) / nv;
         lists = std::max(lists, (size_t)(i1 - i0 + 2 + ctx->row_ptr[i1 + 1] - ctx->row_ptr[i0]) * 4);
     }
     const bool staged = lists <= 32 * 1024;
     if (!staged) lists = 0;
-    a.nres = (int)std::min<int64_t>((cells + grid - 1) / grid,
+    const int64_t most = (cells / cell_unit(nv) + grid - 1) / grid * cell_unit(nv);   // of a CTA
+    a.nres = (int)std::min<int64_t>(most,
                                     (int64_t)((ctx->smem_optin - 1024 - lists) / cell_bytes));
     const size_t smem = a.nres * cell_bytes + lists;
     // window sums by reductions while what a step touches in global memory (both
