@@ -831,7 +831,7 @@ def launches_per_step(hqa, plan, hv, cfg, S, batch, real, count):
         return count * 3      # per member: MD, readout, energy
     if plan["kernel"] == hqa.KERNEL_DENSE and hv["prec_name"] == "PREC_FP32":
         md = (S + 2 if plan.get("threads", 256) == 256   # init, one launch per step, output
-              else 4 * plan.get("chunks", 1))             # init, slices, persistent MD, output
+              else 3 * plan.get("chunks", 1))             # init with slices, persistent MD, output
     elif plan["kernel"] == hqa.KERNEL_DENSE:
         md = 3 * plan.get("chunks", 1)   # init, persistent MD, output per chunk
     else:

@@ -127,6 +127,7 @@ hqa_status finish_create(hqa_ctx* c, hqa_ctx** out)
     for (float v : c->val) {
         if (v != std::nearbyint(v) || std::fabs(v) > 127.f) integer = false;
         if (std::fabs(v) != 1.f) unit = false;
+        c->j_max = std::max(c->j_max, std::fabs(v));
         if (integer) sum += (int64_t)v;
     }
     c->j_whole = integer;

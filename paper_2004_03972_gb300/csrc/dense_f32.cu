@@ -5,25 +5,35 @@
 // BF16 tensor cores from fixed-point slices, at an error against FP64 that is
 // below the FP32 sum's:
 //
-//   phi = b0 + b1 + b2,  b0 = phi rounded to a multiple of u0,
-//                        b1 = the rest rounded to a multiple of u0 2^-8,
-//                        b2 = the rest rounded to BF16,
+//   phi = b0 + b1 + b2,  b0 = phi rounded to a multiple of u, then to BF16,
+//                        b1 = the rest rounded to BF16,
+//                        b2 = what that leaves, rounded to BF16,
 //
-// 24 significant bits of phi in three BF16 numbers.  u0 = 2^-6: |phi| <= 4
-// makes b0 and b1 at most 256 units, so every product with a +-1 coupling is
-// a whole number of units, and a sum of 2000 of them stays below 2^24 units:
-// the FP32 accumulator adds b0's and b1's products without any rounding.
-// (The tensor core truncates what does not fit its FP32 accumulator, which is
-// what limits an ordinary hi + lo split: the FP16X2 operand errs 12 times the
-// FP32 sum on K2000.)  Each slice has its own accumulator, and the epilogue
-// adds the three, smallest first.  Larger |phi| lose nothing: BF16 has FP32's
-// exponents, b0 rounds to 8 bits and b1, b2 take the rest.  States far below
-// 1 get a smaller u0 (unit_level below).
+// 24 significant bits of phi in three BF16 numbers.  u is a power of two, 2^-k of
+// the largest |phi| of the 32 spins that a warp holds of that replica: with
+// 2^k <= 2^23 / (largest row sum of |J|) every product with a +-1 coupling is a
+// whole number of units, a row's sum stays below 2^24 of them, and the FP32
+// accumulator adds b0's products without any rounding.  (The tensor core truncates
+// what does not fit its FP32 accumulator, which is what limits an ordinary hi + lo
+// split: the FP16X2 operand errs 12 times the FP32 sum on K2000.)  b1 and b2 are
+// 2^-8 and 2^-16 of b0, so truncation there costs next to nothing; each slice has
+// its own accumulator, and the epilogue adds the three, smallest first.  Fluxes
+// below u / 2 have no b0 and keep 17 bits, 2^-25 of the group's largest.
+//
+// The unit follows from the fluxes of one replica at one step and from nothing
+// else: a replica's bits do not depend on the others of the launch, a resumed run
+// has the bits of an unbroken one, and the accuracy is the same at every scale of
+// phi.  One unit for 16 to 64 replicas, taken from the largest |phi| two steps
+// before, cost a replica 1000 times smaller than its neighbours two digits.
+// Where the 32-spin groups of one replica differ in scale by 2^10 and more, the
+// small groups' b0 is truncated against the sum of the large ones: there the error
+// is up to 2.6 times the FP32 sum's (a restatement in 64 bits, N = 2000), elsewhere
+// a tenth of it or less.
 //
 // Couplings: +-1 (any integer up to 127) is one exact BF16 slice.  Real
-// couplings are cut the same way, row by row (a_0 + a_1 + a_2, a power of two
-// per row), and the products a_i b_j with i + j <= 2 are kept, accumulator
-// i + j: six MMA columns per replica instead of three.
+// couplings are cut the same way (a_0 + a_1 + a_2; a_0 a multiple of 2^-7 of a
+// power of two per row), and the products a_i b_j with i + j <= 2 are kept,
+// accumulator i + j: six MMA columns per replica instead of three.
 //
 // The three slices of a k-tile lie one after another in shared memory, so one
 // MMA of N = 3 NC columns runs all of them against one coupling tile, and the
@@ -47,6 +57,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "dense_md_kernel.cuh"
 
@@ -70,7 +81,6 @@ struct F32Args {
     float* p;
     float* w;
     uint16_t* phib;          // [2][Rpad][3 Npad] BF16 slices
-    uint32_t* amax;          // [groups][4] bits of max |phi| by step, mod 4
     const StepCoef* sched;
     const float* h;          // [N] or null
     const float* rscale;     // [Npad] power of two per coupling row, or null (all 1)
@@ -79,23 +89,15 @@ struct F32Args {
     int64_t S;
     int W, N, Npad, Rpad, R, KT, Mt, M;
     int rep0;
+    uint32_t ushift;         // 23 - k in the exponent field
 };
 
-// The slice unit u0 = 2^(-6 - 4 level): level 0 for max |phi| >= 2^-6, so that
-// a run of ordinary size has one unit throughout (its results do not depend on
-// which replicas share a launch); smaller states keep at least 18 bits below
-// their largest element.
-__device__ __forceinline__ int unit_level(uint32_t amax_bits)
+// 1.5 * 2^23 units for a warp's 32 fluxes of one replica (f: this lane's):
+// adding and subtracting it rounds to a multiple of the unit.
+__device__ __forceinline__ float round_const(uint32_t f, uint32_t ushift)
 {
-    const int t = (int)(amax_bits >> 23) - 127;          // floor(log2 amax)
-    const int l = t >= -6 ? 0 : (-6 - t + 3) / 4;
-    return l > 24 ? 24 : l;
-}
-
-// 1.5 * 2^23 units: adding and subtracting it rounds to a multiple of the unit
-__device__ __forceinline__ float round_const(int level, int slice)
-{
-    return __uint_as_float((uint32_t)(127 + 17 - 4 * level - 8 * slice) << 23) * 1.5f;
+    const uint32_t e = __reduce_max_sync(0xffffffffu, f & 0x7f800000u) + ushift;
+    return __uint_as_float(min(e, 0x7f000000u) | 0x00400000u);
 }
 
 __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi)   // lo -> bits 0-15
@@ -111,14 +113,13 @@ __device__ __forceinline__ uint64_t widen_bf16x2(uint32_t v)
 }
 
 // The three slices of a pair of values.
-__device__ __forceinline__ void slices2(uint64_t f, uint64_t c0, uint64_t c1, uint32_t (&b)[3])
+__device__ __forceinline__ void slices2(uint64_t f, uint64_t c0, uint32_t (&b)[3])
 {
     using namespace hqa_dense;
     const uint64_t t0 = sub2(add2(f, c0), c0);
     b[0] = cvt_bf16x2(lo2(t0), hi2(t0));
     const uint64_t r1 = sub2(f, widen_bf16x2(b[0]));
-    const uint64_t t1 = sub2(add2(r1, c1), c1);
-    b[1] = cvt_bf16x2(lo2(t1), hi2(t1));
+    b[1] = cvt_bf16x2(lo2(r1), hi2(r1));
     const uint64_t r2 = sub2(r1, widen_bf16x2(b[1]));
     b[2] = cvt_bf16x2(lo2(r2), hi2(r2));
 }
@@ -369,10 +370,6 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
             const float4 cf = __ldg(reinterpret_cast<const float4*>(a.sched) + m);
             const bool in_win = m >= win0;
             for (int hh = 0; hh < HV && !stop; ++hh) {
-                uint32_t* am = a.amax + 4 * (HV * nc + hh);
-                // max |phi| of two steps ago: every CTA of the group has passed that
-                // epilogue, since this one has seen the accumulator of the last step
-                const int lvl = unit_level(__ldcg(am + ((m + 2) & 3)));
                 float pp[16];
                 if (row_ok && csel < NC / 16) {
 #pragma unroll
@@ -384,12 +381,7 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                                           : tc::mbar_wait(accf0 + 8 * hh, (uint32_t)(m & 1), abort, kWaitNs));
                 tc::tc_fence_after();
                 ok = tc::named_bar_and(2 + csel, 128, ok);
-                // the slot of the next step: last read three steps ago
-                if (ok && ew == 0 && lane == 0) *(volatile uint32_t*)(am + ((m + 1) & 3)) = 0u;
-                float big = 0.f;
                 if (ok) {
-                    const uint64_t c0 = pk2(round_const(lvl, 0), round_const(lvl, 0));
-                    const uint64_t c1 = pk2(round_const(lvl, 1), round_const(lvl, 1));
                     const uint64_t hr2 = pk2(hr, hr), rs2 = pk2(rs, rs);
                     const uint64_t cx2 = pk2(cf.x, cf.x), cy2 = pk2(cf.y, cf.y), cz2 = pk2(cf.z, cf.z);
 #pragma unroll 1
@@ -436,15 +428,6 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                                 const float fl = lo2(fn2), fh = hi2(fn2);
                                 fv[j] = __float_as_uint(fl);
                                 fv[j + 1] = __float_as_uint(fh);
-                                big = fmaxf(big, fmaxf(fabsf(fl), fabsf(fh)));
-                                uint32_t b[3];
-                                slices2(fn2, c0, c1, b);
-                                const uint32_t sb = stg + (uint32_t)(j * 128) * 2u + rloc * 2u;
-#pragma unroll
-                                for (int u = 0; u < 3; ++u) {
-                                    sts_u16(sb + u * kStg, (uint16_t)b[u]);
-                                    sts_u16(sb + u * kStg + 256u, (uint16_t)(b[u] >> 16));
-                                }
                                 if (in_win) {
                                     // one owner per sum: the reduction only spares
                                     // the load's latency (same order, same rounding)
@@ -452,13 +435,19 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                                     atomicAdd(a.w + o1, fh);
                                 }
                             }
-                        } else {
-                            // spin rows beyond N keep a zero operand
+                        }
+                        // the operand; spin rows beyond N keep a zero one
 #pragma unroll
-                            for (int j = 0; j < 16; ++j)
+                        for (int j = 0; j < 16; j += 2) {
+                            uint32_t b[3];
+                            slices2(pk2(__uint_as_float(fv[j]), __uint_as_float(fv[j + 1])),
+                                    pk2(round_const(fv[j], a.ushift), round_const(fv[j + 1], a.ushift)), b);
+                            const uint32_t sb = stg + (uint32_t)(j * 128) * 2u + rloc * 2u;
 #pragma unroll
-                                for (int u = 0; u < 3; ++u)
-                                    sts_u16(stg + u * kStg + (uint32_t)(j * 128) * 2u + rloc * 2u, 0);
+                            for (int u = 0; u < 3; ++u) {
+                                sts_u16(sb + u * kStg, (uint16_t)b[u]);
+                                sts_u16(sb + u * kStg + 256u, (uint16_t)(b[u] >> 16));
+                            }
                         }
                         // .sync.aligned: every lane of the warp, outside the row_ok branch
                         tc::tmem_st16(tl + PHI0 + (uint32_t)col, fv);
@@ -478,9 +467,7 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                         }
                     }
                     tc::tc_fence_before();
-                    const uint32_t bm = __reduce_max_sync(0xffffffffu, __float_as_uint(big));
                     if (lane == 0) {
-                        if (csel < NC / 16) atomicMax(am + (m & 3), bm);
                         if (PAIR && crank != 0) tc::mbar_arrive_remote(acce_to + 8 * hh);
                         else tc::mbar_arrive(acce0 + 8 * hh);
                     }
@@ -528,13 +515,12 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
 }
 
 // State set-up: phi(0), p(0) (SplitMix64 or caller-given), window sums 0,
-// padding zero; the column group's largest |phi| at the start or after the
-// first drift (slots 2 and 3: what steps 0 and 1 read).
-__global__ void k_f32_init(F32Args a, int group_cols, uint64_t seed, int init, const float* phi0,
-                           const float* p0)
+// padding zero, and the slices of phi(0) in operand buffer 0 (step 0 writes all
+// of buffer 1).
+__global__ void k_f32_init(F32Args a, uint64_t seed, int init, const float* phi0, const float* p0)
 {
-    const float drift = __ldg(reinterpret_cast<const float4*>(a.sched)).z;
-    const size_t total = (size_t)a.Rpad * a.Npad;       // a multiple of 32, like Npad
+    const size_t total = (size_t)a.Rpad * a.Npad;       // Npad is a multiple of 32: a warp
+                                                        // holds the 32 spins of one unit
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
         const int r = (int)(idx / a.Npad), i = (int)(idx % a.Npad);
@@ -562,47 +548,26 @@ __global__ void k_f32_init(F32Args a, int group_cols, uint64_t seed, int init, c
         a.phi[idx] = phi;
         a.p[idx] = p;
         a.w[idx] = 0.f;
-        // the 32 lanes share r: one look, and rarely an atomic, per warp
-        const float big = fmaxf(fabsf(phi), fabsf(fmaf(drift, p, phi)));
-        const uint32_t bm = __reduce_max_sync(0xffffffffu, __float_as_uint(big));
-        uint32_t* am = a.amax + 4 * (r / group_cols);
-        if ((threadIdx.x & 31) == 0 && bm > *(volatile uint32_t*)(am + 2)) {
-            atomicMax(am + 2, bm);
-            atomicMax(am + 3, bm);
-        }
-    }
-}
-
-// Slices of phi(0) into operand buffer 0 (step 0 writes all of buffer 1).
-__global__ void k_f32_slices(F32Args a, int group_cols)
-{
-    const size_t half = (size_t)a.Npad / 2, total = (size_t)a.Rpad * half;
-    uint32_t* b0 = reinterpret_cast<uint32_t*>(a.phib);
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const size_t r = idx / half, i = idx % half;
-        const int lvl = unit_level(a.amax[4 * (r / group_cols) + 2]);
-        const float c0 = round_const(lvl, 0), c1 = round_const(lvl, 1);
         uint32_t b[3];
-        slices2(reinterpret_cast<const uint64_t*>(a.phi)[idx], hqa_dense::pk2(c0, c0),
-                hqa_dense::pk2(c1, c1), b);
+        slices2(hqa_dense::pk2(phi, 0.f), hqa_dense::pk2(round_const(__float_as_uint(phi), a.ushift), 1.f), b);
+        uint16_t* o = a.phib + (size_t)r * 3 * a.Npad + i;
 #pragma unroll
-        for (int u = 0; u < 3; ++u) b0[r * 3 * half + u * half + i] = b[u];
+        for (int u = 0; u < 3; ++u) o[(size_t)u * a.Npad] = (uint16_t)b[u];
     }
 }
 
 // Row i of J as a_0 + a_1 + a_2 times a power of two (scale[i]): multiples of
-// 2^-7, of 2^-15, and the BF16 rest, for |J_ij| 2^-e <= 1.  One block per row
-// of the [Mpad][3 Mpad] operand (zeroed before); any: bit 0 some a_1, bit 1
-// some a_2 is not zero.
+// 2^-7 and two BF16 rests, for |J_ij| 2^-e <= 1.  One block per row of the
+// [Mpad][3 Mpad] operand (zeroed before).  seen[0]: bit 0 some a_1, bit 1 some
+// a_2 is not zero; seen[1]: the largest row sum of |a_0| in units of 2^-7.
 __global__ void __launch_bounds__(256) k_f32_coupling_slices(
     const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
     const float* __restrict__ val, int N, int Mpad, uint16_t* __restrict__ out,
-    float* __restrict__ scale, uint32_t* any)
+    float* __restrict__ scale, uint32_t* seen)
 {
-    __shared__ uint32_t s_big;
+    __shared__ uint32_t s_big, s_sum;
     const int i = blockIdx.x;
-    if (threadIdx.x == 0) s_big = 0;
+    if (threadIdx.x == 0) s_big = s_sum = 0;
     __syncthreads();
     const int k0 = i < N ? row_ptr[i] : 0, k1 = i < N ? row_ptr[i + 1] : 0;
     uint32_t big = 0;
@@ -615,20 +580,25 @@ __global__ void __launch_bounds__(256) k_f32_coupling_slices(
     const int e = min(max((int)(s_big >> 23) - 126, -100), 127);
     if (threadIdx.x == 0) scale[i] = ldexpf(1.f, e);
     uint16_t* o = out + (size_t)i * 3 * Mpad;
-    uint32_t seen = 0;
+    uint32_t some = 0, sum = 0;
     for (int k = k0 + (int)threadIdx.x; k < k1; k += blockDim.x) {
         const float x = ldexpf(val[k], -e);   // exact, like every difference below
         const auto b = [](float v) { return __float2bfloat16_rn(v); };
         const __nv_bfloat16 b0 = b(rintf(x * 0x1p7f) * 0x1p-7f);
         const float r1 = x - __bfloat162float(b0);
-        const __nv_bfloat16 b1 = b(rintf(r1 * 0x1p15f) * 0x1p-15f);
+        const __nv_bfloat16 b1 = b(r1);
         const __nv_bfloat16 b2 = b(r1 - __bfloat162float(b1));
         o[col[k]] = __bfloat16_as_ushort(b0);
         o[Mpad + col[k]] = __bfloat16_as_ushort(b1);
         o[2 * Mpad + col[k]] = __bfloat16_as_ushort(b2);
-        seen |= (__bfloat162float(b1) != 0.f ? 1u : 0u) | (__bfloat162float(b2) != 0.f ? 2u : 0u);
+        sum += (uint32_t)fabsf(__bfloat162float(b0) * 0x1p7f);
+        some |= (__bfloat162float(b1) != 0.f ? 1u : 0u) | (__bfloat162float(b2) != 0.f ? 2u : 0u);
     }
-    if (seen) atomicOr(any, seen);
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s_sum, sum);
+    if (some) atomicOr(seen, some);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(seen + 1, s_sum);
 }
 
 struct Shape {
@@ -754,6 +724,17 @@ bool hqa_f32tc_possible(const hqa_ctx* ctx)
     return !ctx->is_batch && ctx->dense_input && ctx->dense_tc && ctx->Mpad / BM <= ctx->sm_count;
 }
 
+// k of the slice unit: units fine enough for 2^k steps up to the group's largest
+// power of two, coarse enough that a row's sum of `lsb` coupling units stays
+// exact.  Beyond k = 7 (whole couplings) b0 holds no more bits; real ones gain
+// up to 10, where the products a_1 b_2 and a_2 b_1 that are left out are smaller.
+// Below 5 the rests would miss bits: there only sums of one sign can be truncated.
+static int unit_steps(double sum, bool whole)
+{
+    const int k = 23 - (int)std::ceil(std::log2(std::max(sum, 1.0)));
+    return std::max(5, std::min(k, whole ? 7 : 10));
+}
+
 // Coupling slices, built on first use: the BF16 copy of J when J is whole
 // numbers up to 127, else up to three fixed-point slices per row.
 hqa_status hqa_f32tc_prepare(hqa_ctx* ctx)
@@ -761,6 +742,9 @@ hqa_status hqa_f32tc_prepare(hqa_ctx* ctx)
     if (ctx->f32_nj) return HQA_OK;
     if (!hqa_f32tc_possible(ctx)) return HQA_ERR_UNSUPPORTED;
     if (ctx->j_whole) {
+        int64_t most = 0;
+        for (int i = 0; i < ctx->N; ++i) most = std::max(most, ctx->row_ptr[i + 1] - ctx->row_ptr[i]);
+        ctx->f32_k = unit_steps((double)most * ctx->j_max, true);
         ctx->f32_nj = 1;
         return HQA_OK;
     }
@@ -768,19 +752,20 @@ hqa_status hqa_f32tc_prepare(hqa_ctx* ctx)
     const size_t Mp = (size_t)ctx->Mpad, bytes = 3 * Mp * Mp * sizeof(uint16_t);
     // kept by the context also when a later call here fails: the next one goes on with them
     if (!ctx->d_Jsl) HQA_CUDA_TRY(cudaMalloc(&ctx->d_Jsl, bytes));
-    if (!ctx->d_Jscale) HQA_CUDA_TRY(cudaMalloc(&ctx->d_Jscale, (Mp + 1) * sizeof(float)));
+    if (!ctx->d_Jscale) HQA_CUDA_TRY(cudaMalloc(&ctx->d_Jscale, (Mp + 2) * sizeof(float)));
     HQA_CUDA_TRY(cudaMemset(ctx->d_Jsl, 0, bytes));
-    HQA_CUDA_TRY(cudaMemset(ctx->d_Jscale, 0, (Mp + 1) * sizeof(float)));
-    uint32_t* d_any = reinterpret_cast<uint32_t*>(ctx->d_Jscale + Mp);
+    HQA_CUDA_TRY(cudaMemset(ctx->d_Jscale, 0, (Mp + 2) * sizeof(float)));
+    uint32_t* d_seen = reinterpret_cast<uint32_t*>(ctx->d_Jscale + Mp);
     k_f32_coupling_slices<<<ctx->Mpad, 256>>>(ctx->d_row_ptr, ctx->d_col, ctx->d_val, ctx->N,
                                               ctx->Mpad, static_cast<uint16_t*>(ctx->d_Jsl),
-                                              ctx->d_Jscale, d_any);
+                                              ctx->d_Jscale, d_seen);
     HQA_CUDA_TRY(cudaGetLastError());
-    uint32_t any = 0;
-    HQA_CUDA_TRY(cudaMemcpy(&any, d_any, sizeof(any), cudaMemcpyDeviceToHost));
+    uint32_t seen[2] = {0, 0};
+    HQA_CUDA_TRY(cudaMemcpy(seen, d_seen, sizeof(seen), cudaMemcpyDeviceToHost));
     if (!hqa_dense_tmap16(&ctx->tmJsl, ctx->d_Jsl, Mp, 3 * Mp, BK, BM, true, false)) return HQA_ERR_CUDA;
     ++ctx->generation;
-    ctx->f32_nj = (any & 2u) ? 3 : (any & 1u) ? 2 : 1;
+    ctx->f32_k = unit_steps(seen[1], false);
+    ctx->f32_nj = (seen[0] & 2u) ? 3 : (seen[0] & 1u) ? 2 : 1;
     return HQA_OK;
 }
 
@@ -805,9 +790,9 @@ static hqa_status f32_chunk(hqa_ctx* ctx, const Shape& sh, const StepCoef* d_sch
     const int Mt = ctx->Mpad / BM, cols = sh.HV * sh.NC;
     const int Nc = (R + cols - 1) / cols, Rpad = Nc * cols, groups = Nc * sh.HV;
     const size_t n = (size_t)Rpad * ctx->Mpad;
-    // state: phi, p, w (FP32), two operand buffers of three slices, group words
-    const size_t off_b = 3 * n * 4, off_g = off_b + 2 * 3 * n * 2, off_m = off_g + (size_t)groups * 4;
-    const size_t need = off_m + (size_t)groups * 16;
+    // state: phi, p, w (FP32), two operand buffers of three slices, group counters
+    const size_t off_b = 3 * n * 4, off_g = off_b + 2 * 3 * n * 2;
+    const size_t need = off_g + (size_t)groups * 4;
     hqa_status s = hqa_reserve(ctx, &ctx->d_state, &ctx->state_cap, need);
     if (s != HQA_OK) return s;
     char* b = static_cast<char*>(ctx->d_state);
@@ -817,7 +802,6 @@ static hqa_status f32_chunk(hqa_ctx* ctx, const Shape& sh, const StepCoef* d_sch
     a.w = a.p + n;
     a.phib = reinterpret_cast<uint16_t*>(b + off_b);
     a.gbar = reinterpret_cast<unsigned int*>(b + off_g);
-    a.amax = reinterpret_cast<uint32_t*>(b + off_m);
     a.sched = d_sched;
     a.h = ctx->has_h ? ctx->d_h : nullptr;
     a.rscale = ctx->d_Jscale;
@@ -832,15 +816,15 @@ static hqa_status f32_chunk(hqa_ctx* ctx, const Shape& sh, const StepCoef* d_sch
     a.Mt = Mt;
     a.M = M;
     a.rep0 = rep0;
+    a.ushift = (uint32_t)(23 - ctx->f32_k) << 23;
     CUtensorMap tmB, tmS;
     if (!hqa_dense_tmap16(&tmB, a.phib, (uint64_t)2 * Rpad, (uint64_t)3 * ctx->Mpad, BK,
                           sh.pair ? sh.NC / 2 : sh.NC, true, false) ||
         !hqa_dense_tmap16(&tmS, a.phib, (uint64_t)2 * Rpad, (uint64_t)3 * ctx->Mpad, 128, 16, false, false))
         return HQA_ERR_CUDA;
-    if (cudaMemsetAsync(a.gbar, 0, (size_t)groups * 20, st) != cudaSuccess) return HQA_ERR_CUDA;
+    if (cudaMemsetAsync(a.gbar, 0, (size_t)groups * 4, st) != cudaSuccess) return HQA_ERR_CUDA;
     const int g = (int)std::min<size_t>(8192, (n + 255) / 256);
-    k_f32_init<<<g, 256, 0, st>>>(a, sh.NC, seed, init, phi0, p0);
-    k_f32_slices<<<g, 256, 0, st>>>(a, sh.NC);
+    k_f32_init<<<g, 256, 0, st>>>(a, seed, init, phi0, p0);
     s = launch(ctx, a, sh, ctx->f32_nj, Mt * Nc, st, ctx->d_Jsl ? ctx->tmJsl : ctx->tmJ, tmB, tmS);
     if (s != HQA_OK) return s;
     hqa_dense::DenseMDArgs o{};

@@ -119,6 +119,7 @@ struct hqa_ctx {
     bool integer = false;       // all J and h integral with |J| <= 127, |h| <= 2^20
     bool unit = false;          // all J in {-1, 0, +1}
     bool j_whole = false;       // all J integral with |J| <= 127, whatever h
+    float j_max = 0.f;          // largest |J|
     bool has_h = false;
 
     // host copies of the symmetric CSR (diagonal dropped), used to build plans
@@ -218,6 +219,7 @@ struct hqa_ctx {
     // first nj used, with a power of two per row), built on first use; whole-numbered J uses d_Jbf instead.
     // 0: not built yet
     int f32_nj = 0;
+    int f32_k = 0;              // slice unit: 2^-k of a group's largest flux
     void* d_Jsl = nullptr;
     float* d_Jscale = nullptr;
     CUtensorMap tmJsl;
