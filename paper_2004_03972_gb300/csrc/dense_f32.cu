@@ -85,6 +85,7 @@ struct F32Args {
     const float* h;          // [N] or null
     const float* rscale;     // [Npad] power of two per coupling row, or null (all 1)
     unsigned int* gbar;      // [groups] arrival counters
+    uint32_t* tiny;          // not 0: window sums without reductions (hqa_tiny_state)
     uint32_t* status;
     int64_t S;
     int W, N, Npad, Rpad, R, KT, Mt, M;
@@ -350,6 +351,7 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
         const float rs = a.rscale ? a.rscale[row] : 1.f;
         const int mhalf = (a.M - 2) / 2;
         const int64_t win0 = a.S - (int64_t)a.W;
+        const bool tiny = __ldcg(a.tiny) != 0u;
         const uint32_t tl = tmem + ((uint32_t)(32 * quarter) << 16);
         const uint32_t rloc = (uint32_t)(32 * quarter + lane);
         const uint32_t acce_to = (PAIR && crank != 0) ? tc::mapa(acce0, 0) : acce0;
@@ -368,7 +370,7 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
         bool stop = false;
         for (int64_t m = 0; m < a.S && !stop; ++m) {
             const float4 cf = __ldg(reinterpret_cast<const float4*>(a.sched) + m);
-            const bool in_win = m >= win0;
+            const bool in_win = m >= win0 && !tiny, plain_win = m >= win0 && tiny;
             for (int hh = 0; hh < HV && !stop; ++hh) {
                 float pp[16];
                 if (row_ok && csel < NC / 16) {
@@ -429,11 +431,15 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                                 fv[j] = __float_as_uint(fl);
                                 fv[j + 1] = __float_as_uint(fh);
                                 if (in_win) {
-                                    // one owner per sum: the reduction only spares
-                                    // the load's latency (same order, same rounding)
-                                    atomicAdd(a.w + o0, fl);
-                                    atomicAdd(a.w + o1, fh);
+                                    win_add(a.w + o0, fl);
+                                    win_add(a.w + o1, fh);
                                 }
+                            }
+                            if (plain_win) {
+                                float f[16];
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(fv[j]);
+                                hqa_win_plain16(a.w + (size_t)(n0 + col) * a.Npad + row, a.Npad, f);
                             }
                         }
                         // the operand; spin rows beyond N keep a zero one
@@ -545,6 +551,7 @@ __global__ void k_f32_init(F32Args a, uint64_t seed, int init, const float* phi0
                 }
             }
         }
+        if (init == HQA_INIT_GIVEN && r < a.R && i < a.N && hqa_tiny_state(phi, p)) *a.tiny = 1u;
         a.phi[idx] = phi;
         a.p[idx] = p;
         a.w[idx] = 0.f;
@@ -790,9 +797,10 @@ static hqa_status f32_chunk(hqa_ctx* ctx, const Shape& sh, const StepCoef* d_sch
     const int Mt = ctx->Mpad / BM, cols = sh.HV * sh.NC;
     const int Nc = (R + cols - 1) / cols, Rpad = Nc * cols, groups = Nc * sh.HV;
     const size_t n = (size_t)Rpad * ctx->Mpad;
-    // state: phi, p, w (FP32), two operand buffers of three slices, group counters
+    // state: phi, p, w (FP32), two operand buffers of three slices, group counters,
+    // the mark of a tiny state
     const size_t off_b = 3 * n * 4, off_g = off_b + 2 * 3 * n * 2;
-    const size_t need = off_g + (size_t)groups * 4;
+    const size_t need = off_g + ((size_t)groups + 1) * 4;
     hqa_status s = hqa_reserve(ctx, &ctx->d_state, &ctx->state_cap, need);
     if (s != HQA_OK) return s;
     char* b = static_cast<char*>(ctx->d_state);
@@ -802,6 +810,7 @@ static hqa_status f32_chunk(hqa_ctx* ctx, const Shape& sh, const StepCoef* d_sch
     a.w = a.p + n;
     a.phib = reinterpret_cast<uint16_t*>(b + off_b);
     a.gbar = reinterpret_cast<unsigned int*>(b + off_g);
+    a.tiny = a.gbar + groups;
     a.sched = d_sched;
     a.h = ctx->has_h ? ctx->d_h : nullptr;
     a.rscale = ctx->d_Jscale;
@@ -822,7 +831,7 @@ static hqa_status f32_chunk(hqa_ctx* ctx, const Shape& sh, const StepCoef* d_sch
                           sh.pair ? sh.NC / 2 : sh.NC, true, false) ||
         !hqa_dense_tmap16(&tmS, a.phib, (uint64_t)2 * Rpad, (uint64_t)3 * ctx->Mpad, 128, 16, false, false))
         return HQA_ERR_CUDA;
-    if (cudaMemsetAsync(a.gbar, 0, (size_t)groups * 4, st) != cudaSuccess) return HQA_ERR_CUDA;
+    if (cudaMemsetAsync(a.gbar, 0, ((size_t)groups + 1) * 4, st) != cudaSuccess) return HQA_ERR_CUDA;
     const int g = (int)std::min<size_t>(8192, (n + 255) / 256);
     k_f32_init<<<g, 256, 0, st>>>(a, seed, init, phi0, p0);
     s = launch(ctx, a, sh, ctx->f32_nj, Mt * Nc, st, ctx->d_Jsl ? ctx->tmJsl : ctx->tmJ, tmB, tmS);

@@ -472,9 +472,9 @@ static hqa_status dense_md_chunk(hqa_ctx* ctx, bool wide, const StepCoef* d_sche
     const size_t n = (size_t)Rpad * Npad;
     const int kseg = kseg_of(ctx, prec);
     const size_t nb = (size_t)kseg * n;   // operand elements per buffer
-    // state: phi, p, w (FP32), two 16-bit operand buffers, 2 Nc counters
+    // state: phi, p, w (FP32), two 16-bit operand buffers, 2 Nc counters, the mark of a tiny state
     const size_t off_p = n * 4, off_w = 2 * n * 4, off_b = 3 * n * 4, off_g = off_b + 2 * nb * 2;
-    const size_t need = off_g + (size_t)2 * Nc * sizeof(unsigned int);
+    const size_t need = off_g + ((size_t)2 * Nc + 1) * sizeof(unsigned int);
     hqa_status s = hqa_reserve(ctx, &ctx->d_state, &ctx->state_cap, need);
     if (s != HQA_OK) return s;
     char* b = static_cast<char*>(ctx->d_state);
@@ -484,6 +484,7 @@ static hqa_status dense_md_chunk(hqa_ctx* ctx, bool wide, const StepCoef* d_sche
     a.w = reinterpret_cast<float*>(b + off_w);
     a.phib = reinterpret_cast<uint16_t*>(b + off_b);
     a.gbar = reinterpret_cast<unsigned int*>(b + off_g);
+    a.tiny = a.gbar + 2 * Nc;
     a.sched = d_sched;
     a.h = ctx->has_h ? ctx->d_h : nullptr;
     a.status = ctx->d_status;
@@ -516,11 +517,11 @@ static hqa_status dense_md_chunk(hqa_ctx* ctx, bool wide, const StepCoef* d_sche
         return HQA_ERR_CUDA;
     const CUtensorMap& tmA = f16 ? (kseg == 3 ? ctx->tmJh3 : ctx->tmJh)
                                  : (kseg == 3 ? ctx->tmJ3 : ctx->tmJ);
+    if (cudaMemsetAsync(a.gbar, 0, ((size_t)2 * Nc + 1) * sizeof(unsigned int), st) != cudaSuccess)
+        return HQA_ERR_CUDA;
     const int g = (int)std::min<size_t>(8192, (n + 255) / 256);
     if (f16) hqa_dense::k_dense_init<true><<<g, 256, 0, st>>>(a, seed, init, phi0, p0, kseg);
     else hqa_dense::k_dense_init<false><<<g, 256, 0, st>>>(a, seed, init, phi0, p0, kseg);
-    if (cudaMemsetAsync(a.gbar, 0, (size_t)2 * Nc * sizeof(unsigned int), st) != cudaSuccess)
-        return HQA_ERR_CUDA;
     s = wide ? hqa_wide_launch(ctx, a, kseg, f16, st, tmA, tmB)
       : f16 ? hqa_dense::dense_md_dispatch<true>(ctx, a, NH, kseg, grid, st, tmA, tmB, tmS)
             : hqa_dense::dense_md_dispatch<false>(ctx, a, NH, kseg, grid, st, tmA, tmB, tmS);

@@ -82,7 +82,8 @@ constexpr bool kTmaStore = true;
 constexpr uint32_t kStgBytes = 16 * 128 * 2;   // one staging tile [16 replicas][128 spins]
 
 // One window sum: its only owner adds once per step, so the reduction gives
-// the load-add-store's result (bitwise) without waiting for the load.  K2000 x
+// the load-add-store's result without waiting for the load (bitwise outside the
+// states that hqa_tiny_state marks, which do not come here).  K2000 x
 // 4096, 40 steps inside the window: FP16X2 2.82 -> 1.99 ms, BF16 2.36 -> 1.56 ms;
 // outside the window a step is unchanged (43 and 30 us).
 __device__ __forceinline__ void win_add(float* w, float v) { atomicAdd(w, v); }
@@ -139,6 +140,7 @@ struct DenseMDArgs {
     const StepCoef* sched;
     const float* h;          // [N] or null
     unsigned int* gbar;      // [2 Nc] arrival counters
+    uint32_t* tiny;          // not 0: window sums without reductions (hqa_tiny_state)
     uint32_t* status;
     int64_t S;
     int W, N, Npad, Rpad, R, KT, Mt, M;
@@ -430,6 +432,7 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
         const float hr = (a.h && row_ok) ? 2.f * a.h[row] : 0.f;
         const int mhalf = (a.M - 2) / 2;
         const int64_t win0 = a.S - (int64_t)a.W;
+        const bool tiny = __ldcg(a.tiny) != 0u;
         const uint32_t tl = (uint32_t)(32 * quarter) << 16;   // this warp's TMEM lanes
         const uint32_t rloc = (uint32_t)(32 * quarter + lane);  // row within the tile
         // PAIR, odd CTA: accumulators are released on the even CTA's barrier
@@ -463,7 +466,7 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
         bool stop = false;
         for (int64_t m = 0; m < a.S && !stop; ++m) {
             const float4 cf = __ldg(reinterpret_cast<const float4*>(a.sched) + m);
-            const bool in_win = m >= win0;
+            const bool in_win = m >= win0 && !tiny, plain_win = m >= win0 && tiny;
             const int Kb = KSEG * a.Npad;   // operand row: [hi], [hi | lo] or [hi | hi | lo]
             uint16_t* nb = a.phib + (size_t)((m + 1) & 1) * a.Rpad * Kb;
             bool ok = true;
@@ -591,6 +594,12 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
                                 if constexpr (KSEG != 1) sts_u16(sb + kStgBytes, 0);
                             }
                         }
+                        if (plain_win && row_ok) {
+                            float f[16];
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(fv[j]);
+                            hqa_win_plain16(a.w + (size_t)(n0 + col) * a.Npad + row, a.Npad, f);
+                        }
                         // .sync.aligned: every lane of the warp, outside the row_ok branch
                         tc::tmem_st16(tmem + tl + (uint32_t)(2 * NH + col), fv);
                         tc::tmem_wait_st();
@@ -653,7 +662,10 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
                                     nb[ob + 2 * a.Npad] = cvt16<F16>(fs - from16<F16>(hi));
                                 }
                                 if (in_win) win_add(a.w + (size_t)(n0 + col + j) * a.Npad + row, fn);
+                                phl[j] = fn;
                             }
+                            if (plain_win)
+                                hqa_win_plain16(a.w + (size_t)(n0 + col) * a.Npad + row, a.Npad, phl);
                         }
                         // .sync.aligned: every lane of the warp, outside the row_ok branch
                         tc::tmem_st16(tmem + tl + (uint32_t)(2 * NH + col), pv);
@@ -702,7 +714,10 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
                                     nb[ob + 2 * a.Npad] = cvt16<F16>(fs - from16<F16>(hi));
                                 }
                                 if (in_win) win_add(a.w + o, fn);
+                                ph[j] = fn;
                             }
+                            if (plain_win)
+                                hqa_win_plain16(a.w + (size_t)rbase * a.Npad + row, a.Npad, ph);
                         }
                         if (more) {
 #pragma unroll
@@ -812,6 +827,7 @@ __global__ void k_dense_init(DenseMDArgs a, uint64_t seed, int init, const float
                 }
             }
         }
+        if (init == HQA_INIT_GIVEN && r < a.R && i < a.N && hqa_tiny_state(phi, p)) *a.tiny = 1u;
         a.phi[idx] = phi;
         a.p[idx] = p;
         a.w[idx] = 0.f;

@@ -227,6 +227,7 @@ k_dense_wide(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CU
         const uint32_t acce_to = crank != 0 ? tc::mapa(acce0, 0) : acce0;
         const int mhalf = (a.M - 2) / 2;
         const int64_t win0 = a.S - (int64_t)a.W;
+        const bool tiny = __ldcg(a.tiny) != 0u;
         const int Kb = KSEG * a.Npad;         // operand row: [hi], [hi | lo] or [hi | hi | lo]
         bool stop = false;
         uint32_t i = 0;
@@ -235,7 +236,7 @@ k_dense_wide(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CU
             const int u = (int)(g % U), cb = u / w.RT, rt = u % w.RT;
             const uint32_t b = i & 1u;
             const float4 cf = __ldg(reinterpret_cast<const float4*>(a.sched) + m);
-            const bool in_win = m >= win0;
+            const bool in_win = m >= win0 && !tiny, plain_win = m >= win0 && tiny;
             const int row = rt * 2 * BM + (int)crank * BM + 32 * quarter + lane;
             const bool row_ok = row < a.N;
             const float hr = (a.h && row_ok) ? 2.f * __ldg(a.h + row) : 0.f;
@@ -288,7 +289,9 @@ k_dense_wide(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CU
                                 nb[ob + 2 * a.Npad] = cvt16<F16>(fs - from16<F16>(hi));
                             }
                             if (in_win) win_add(a.w + o, fn);
+                            ph[j] = fn;
                         }
+                        if (plain_win) hqa_win_plain16(a.w + (size_t)rbase * a.Npad + row, a.Npad, ph);
                     }
                     if (more) {
 #pragma unroll

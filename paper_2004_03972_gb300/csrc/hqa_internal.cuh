@@ -45,6 +45,28 @@ __device__ __forceinline__ float pot_pow(float phi, float phi2, int mhalf)
     return pw;
 }
 
+// Reductions on global memory flush subnormal operands and results, which a window
+// sum can only meet where the flux stays below 2^-100 in the window: larger terms
+// make every sum zero or normal.  A state that starts with such a spin (phi and p
+// below 2^-80; given states only, else p = +-1) is marked at set-up, and the run
+// then sums by load, add and store.  The mark is one word, so that a step pays no
+// test per element (one in the update cost K2000 FP16 3 %, one after it K2000
+// FP16X2 2 %).
+__device__ __forceinline__ bool hqa_tiny_state(float phi, float p)
+{
+    return fabsf(phi) < 0x1p-80f && fabsf(p) < 0x1p-80f;
+}
+
+// 16 window sums without reductions: volatile, so past L1, one after another.
+__device__ __forceinline__ void hqa_win_plain16(float* w, size_t stride, const float (&v)[16])
+{
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        volatile float* o = w + j * stride;
+        *o = *o + v[j];
+    }
+}
+
 // One step of the kick/drift coefficient table (see hqa_run).
 struct StepCoef {
     float kA;  // c_j h alpha(j dt) M       multiplies phi^(M-1)

@@ -56,7 +56,7 @@ struct StreamArgs {
     float* phi;            // [N][Rpad] FP32 master (BF16 operand only)
     float* p;
     float* w;
-    unsigned int* bar;     // grid barrier arrival counter
+    unsigned int* bar;     // grid barrier arrival counter; [1] not 0: a tiny state
     uint32_t* status;
     int64_t S;
     int W, N, Rpad, M;
@@ -290,6 +290,8 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
     const int i0 = (int)(first / nv), v0 = (int)(first % nv);
     const int di = kMDThreads / nv, dv = kMDThreads % nv;
     const int64_t win0 = a.S - (int64_t)a.W;
+    __shared__ uint32_t s_tiny;   // marked by the set-up; in shared memory, as a register costs 1 %
+    if (threadIdx.x == 0) s_tiny = __ldcg(a.bar + 1);
     const int mhalf = (a.M - 2) / 2;
     // global address of plane q of the cell at offset o
     const auto gplane = [&](int q, size_t o) {
@@ -311,8 +313,8 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
             s_off[k] = (rows ? a.row_ptr[rowA + k] : 0) - kA;
         for (int k = kA + (int)threadIdx.x; k < kB; k += kMDThreads)
             s_ent[k - kA] = (uint32_t)a.col[k] | (a.val[k] < 0 ? 0x80000000u : 0u);
-        __syncthreads();
     }
+    __syncthreads();
     for (int64_t m = 0; m < a.S; ++m) {
         const float4 cf = __ldg(reinterpret_cast<const float4*>(a.sched) + m);
         const void* cur = (m & 1) ? a.op1 : a.op0;
@@ -352,12 +354,13 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
 #pragma unroll
             for (int q = 0; q < NP; ++q) put4(res ? st + q * a.nres + l : gplane(q, o), sv + 4 * q);
             // one owner per window sum: the reduction gives the load, add and
-            // store's result without waiting for the load
+            // store's result without waiting for the load (bitwise outside the
+            // states that hqa_tiny_state marks)
             if (in_win) {
 #pragma unroll
                 for (int e = 0; e < V; e += 4) {
                     float4* w = reinterpret_cast<float4*>(a.w + o + e);
-                    if (a.wred) {
+                    if (a.wred && *(volatile uint32_t*)&s_tiny == 0u) {
                         atomicAdd(w, make_float4(fn[e], fn[e + 1], fn[e + 2], fn[e + 3]));
                     } else {
                         float4 q = *w;
@@ -434,6 +437,7 @@ k_stream_init(StreamArgs a, int R, uint64_t seed, int init, const float* phi0, c
                 if (init == HQA_INIT_GIVEN) {
                     f = phi0[(size_t)r * a.N + i];
                     q = p0[(size_t)r * a.N + i];
+                    if (hqa_tiny_state(f, q)) a.bar[1] = 1u;
                 } else {
                     uint64_t z = seed + (c + 1ull) * 0x9E3779B97F4A7C15ull;  // SplitMix64
                     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -581,9 +585,9 @@ hqa_status hqa_stream_launch_md(hqa_ctx* ctx, int prec, const StepCoef* d_sched,
         return (unsigned)std::min<int64_t>(
             65536, (int64_t)((ctx->N + kTile - 1) / kTile) * ((reps + kTile - 1) / kTile));
     };
+    if (cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned int), st) != cudaSuccess) return HQA_ERR_CUDA;
     if (bf16) k_stream_init<true><<<tiles(a.Rpad), tile, 0, st>>>(a, R, seed, init, phi0, p0);
     else k_stream_init<false><<<tiles(a.Rpad), tile, 0, st>>>(a, R, seed, init, phi0, p0);
-    if (cudaMemsetAsync(a.bar, 0, sizeof(unsigned int), st) != cudaSuccess) return HQA_ERR_CUDA;
     // persistent grid: every CTA co-resident (the per-step barrier waits on all of
     // them), one per SM; small problems take fewer, at least a quarter full
     const int64_t cells = (int64_t)ctx->N * (a.Rpad / (bf16 ? 8 : 4));
