@@ -170,7 +170,9 @@ void hqa_run_opts_default(hqa_run_opts* o);
 enum {
     HQA_J_BF16 = 1u << 0, /* BF16 tensor-core operand (always built for the tcgen05 path) */
     HQA_J_FP16 = 1u << 1, /* FP16 tensor-core operand, J * 2^10 (HQA_PREC_FP16 / FP16X2) */
-    HQA_J_FP32 = 1u << 2, /* FP32 operand of the CUDA-core dense GEMM (HQA_PREC_FP32) */
+    HQA_J_FP32 = 1u << 2, /* operands of HQA_PREC_FP32: J in FP32 (local fields, and runs
+                             beyond N = 19456), and for real J the three BF16 slices
+                             that the runs multiply (6 bytes a coupling) */
     HQA_J_FP8 = 1u << 3   /* FP8 E4M3: not provided (HQA_ERR_UNSUPPORTED).  The kind::f16
                              MMA needs both operands in the same 16-bit format, and an
                              FP8 MMA would need phi in FP8 (3 significant bits); widening

@@ -597,7 +597,9 @@ hqa_status hqa_create_dense(int32_t N, const float* J, const float* h, uint32_t 
     if (s != HQA_OK) return s;
     s = hqa_dense_setup(c, J);
     if (s == HQA_OK && (flags & HQA_J_FP16)) s = hqa_dense_prepare(c, HQA_PREC_FP16);
+    // the fields read the FP32 copy, the runs the slices
     if (s == HQA_OK && (flags & HQA_J_FP32)) s = hqa_simt_prepare(c);
+    if (s == HQA_OK && (flags & HQA_J_FP32) && hqa_f32tc_possible(c)) s = hqa_f32tc_prepare(c);
     if (s != HQA_OK) {
         hqa_destroy(c);
         *out = nullptr;
@@ -876,8 +878,7 @@ hqa_status hqa_plan_query(hqa_ctx* ctx, int32_t replicas, const hqa_run_opts* op
     if (s != HQA_OK) return s;
     if (dense == 2 && hqa_f32tc_possible(ctx)) {
         int rb = 0, grid = 0, C = 1;
-        s = hqa_f32tc_plan(ctx, replicas, &rb, &grid, &C);
-        if (s != HQA_OK) return s;
+        hqa_f32tc_plan(ctx, replicas, &rb, &grid, &C);
         out->kernel = HQA_KERNEL_DENSE;
         out->replicas_per_block = rb;
         out->blocks = grid;

@@ -58,6 +58,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "dense_md_kernel.cuh"
 
@@ -563,6 +564,14 @@ __global__ void k_f32_init(F32Args a, uint64_t seed, int init, const float* phi0
     }
 }
 
+// The power of two that bounds a row whose largest |J| has these bits: below 2^e,
+// with e kept where the scale and the slices stay normal numbers.
+__host__ __device__ inline int row_exponent(uint32_t bits)
+{
+    const int e = (int)(bits >> 23) - 126;
+    return e < -100 ? -100 : e > 127 ? 127 : e;
+}
+
 // Row i of J as a_0 + a_1 + a_2 times a power of two (scale[i]): multiples of
 // 2^-7 and two BF16 rests, for |J_ij| 2^-e <= 1.  One block per row of the
 // [Mpad][3 Mpad] operand (zeroed before).  seen[0]: bit 0 some a_1, bit 1 some
@@ -583,8 +592,7 @@ __global__ void __launch_bounds__(256) k_f32_coupling_slices(
     big = __reduce_max_sync(0xffffffffu, big);
     if ((threadIdx.x & 31) == 0) atomicMax(&s_big, big);
     __syncthreads();
-    // the largest is below 2^e; the scale and the slices stay normal numbers
-    const int e = min(max((int)(s_big >> 23) - 126, -100), 127);
+    const int e = row_exponent(s_big);
     if (threadIdx.x == 0) scale[i] = ldexpf(1.f, e);
     uint16_t* o = out + (size_t)i * 3 * Mpad;
     uint32_t some = 0, sum = 0;
@@ -706,6 +714,32 @@ hqa_status launch(hqa_ctx* ctx, const F32Args& a, const Shape& s, int nj, int gr
     return launch_nj<16, 1>(ctx, a, nj, s.pair, grid, st, tmJ, tmB, tmS);
 }
 
+// Whether J is one BF16 slice, as k_f32_coupling_slices will find it, without
+// building anything: a plan query needs to know, also during a capture.  The first
+// coupling that is not a multiple of 2^-7 of its row's power of two ends the look.
+bool one_slice(hqa_ctx* ctx)
+{
+    if (ctx->f32_nj) return ctx->f32_nj == 1;
+    if (ctx->f32_one < 0) {
+        ctx->f32_one = 1;
+        for (int i = 0; i < ctx->N && ctx->f32_one && !ctx->j_whole; ++i) {
+            float big = 0.f;
+            for (int64_t k = ctx->row_ptr[i]; k < ctx->row_ptr[i + 1]; ++k)
+                big = std::max(big, std::fabs(ctx->val[k]));
+            uint32_t bits;
+            std::memcpy(&bits, &big, 4);
+            for (int64_t k = ctx->row_ptr[i]; k < ctx->row_ptr[i + 1]; ++k) {
+                const float x = std::ldexp(ctx->val[k], 7 - row_exponent(bits));
+                if (x != std::rint(x)) {
+                    ctx->f32_one = 0;
+                    break;
+                }
+            }
+        }
+    }
+    return ctx->f32_one == 1;
+}
+
 // Replicas one launch takes: as many column groups as fit next to the row
 // tiles with one CTA per SM.
 int chunk_replicas(const hqa_ctx* ctx, const Shape& s)
@@ -715,9 +749,9 @@ int chunk_replicas(const hqa_ctx* ctx, const Shape& s)
 
 // The narrowest tile that runs all replicas in one launch (a narrow tile
 // spreads few replicas over more SMs), else the widest.
-Shape pick_shape(const hqa_ctx* ctx, int R, int nj)
+Shape pick_shape(hqa_ctx* ctx, int R)
 {
-    const bool pairs = nj == 1 && (ctx->Mpad / BM) % 2 == 0;
+    const bool pairs = one_slice(ctx) && (ctx->Mpad / BM) % 2 == 0;
     const Shape c[4] = {{16, 1, false}, {32, 1, false}, {64, 1, pairs}, {64, 2, pairs}};
     for (int k = 0; k < 3; ++k)
         if (R <= chunk_replicas(ctx, c[k])) return c[k];
@@ -776,17 +810,14 @@ hqa_status hqa_f32tc_prepare(hqa_ctx* ctx)
     return HQA_OK;
 }
 
-hqa_status hqa_f32tc_plan(hqa_ctx* ctx, int32_t R, int* rb, int* grid, int* chunks)
+void hqa_f32tc_plan(hqa_ctx* ctx, int32_t R, int* rb, int* grid, int* chunks)
 {
-    hqa_status s = hqa_f32tc_prepare(ctx);
-    if (s != HQA_OK) return s;
-    const Shape sh = pick_shape(ctx, R, ctx->f32_nj);
+    const Shape sh = pick_shape(ctx, R);
     const int Rc = chunk_replicas(ctx, sh);
     *chunks = (R + Rc - 1) / Rc;
     const int per = (R + *chunks - 1) / *chunks;
     *rb = sh.HV * sh.NC;
     *grid = ctx->Mpad / BM * ((per + *rb - 1) / *rb);
-    return HQA_OK;
 }
 
 static hqa_status f32_chunk(hqa_ctx* ctx, const Shape& sh, const StepCoef* d_sched, int64_t S,
@@ -856,7 +887,7 @@ hqa_status hqa_f32tc_launch_md(hqa_ctx* ctx, const StepCoef* d_sched, int64_t S,
 {
     hqa_status s = hqa_f32tc_prepare(ctx);
     if (s != HQA_OK) return s;
-    const Shape sh = pick_shape(ctx, R, ctx->f32_nj);
+    const Shape sh = pick_shape(ctx, R);
     const int most = chunk_replicas(ctx, sh);
     const int C = (R + most - 1) / most, Rc = (R + C - 1) / C;
     for (int r0 = 0; r0 < R; r0 += Rc) {

@@ -242,6 +242,7 @@ struct hqa_ctx {
     // 0: not built yet
     int f32_nj = 0;
     int f32_k = 0;              // slice unit: 2^-k of a group's largest flux
+    int f32_one = -1;           // 1: one slice holds J, 0: not, -1: not looked at yet
     void* d_Jsl = nullptr;
     float* d_Jscale = nullptr;
     CUtensorMap tmJsl;
@@ -342,7 +343,7 @@ bool hqa_dense_tmap16(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t c
 // dense_f32.cu: the FP32 dense path on the tensor cores (fixed-point slices)
 bool hqa_f32tc_possible(const hqa_ctx* ctx);
 hqa_status hqa_f32tc_prepare(hqa_ctx* ctx);
-hqa_status hqa_f32tc_plan(hqa_ctx* ctx, int32_t R, int* rb, int* grid, int* chunks);
+void hqa_f32tc_plan(hqa_ctx* ctx, int32_t R, int* rb, int* grid, int* chunks);
 hqa_status hqa_f32tc_launch_md(hqa_ctx* ctx, const StepCoef* d_sched, int64_t S, int32_t W,
                                int32_t R, uint64_t seed, int init, const float* phi0,
                                const float* p0, int M, float* phi_out, float* p_out,
