@@ -478,12 +478,27 @@ __global__ void __launch_bounds__(kEnumThreads) k_sub_enum16_arg(const SubPrep* 
 //     in s_j and goes into j's field; its sign follows from s_j afterwards.
 // What is left splits into connected components, each enumerated by the CTA in
 // Gray order, 2^(c - 8) steps per thread.  A component of more than 12 spins is
-// solved here only when it is at least 4 spins smaller than the whole problem:
-// a step here takes about ten times the packed walk's 1.2 instructions per
-// configuration, so up to there this is the shorter way; the walks get the rest
-// (complete graphs).  ER800 x 1024, n = 24 (16.8 M configurations, of which the
-// reduction leaves a few hundred): 3.1 ms of walks before, 21 us.
+// solved here only when that is the shorter way (enum_here); the walks get the
+// rest.  ER800 x 1024, n = 24 (16.8 M configurations, of which the reduction
+// leaves a few hundred): 3.1 ms of walks before, 21 us.
 constexpr int kTieShift = 33;
+
+// Whether this CTA's walk of c spins, 2^(c - 8) steps one after another, takes
+// less time than the packed walk of all 2^n configurations over the whole GPU.
+// A step takes 59 ns while every replica has an SM of its own and 0.3 ns times
+// the replicas beyond; the packed walk 1.43e-4 ns per configuration and, from 2^22
+// of them on, 16 us of fixed latency.  Complete graphs of c spins, this walk / the
+// packed one, us: n = 24, one replica, c = 16 70 / 78, 18 115 / 74; n = 30, one
+// replica, c = 18 116 / 240, 20 296 / 234, 26 15400 / 230; n = 30, 64 replicas,
+// c = 25 7757 / 9679, 26 15620 / 9660; n = 24, 1024 replicas, c = 20 1237 / 3610.
+__device__ __forceinline__ bool enum_here(int c, int n, int replicas)
+{
+    if (c <= 12) return true;
+    if (c > n - 4) return false;
+    const float configs = ldexpf((float)replicas, n);
+    const float packed_ns = (configs >= 0x1p22f ? 16000.f : 3000.f) + 1.43e-4f * configs;
+    return ldexpf(fmaxf(59.f, 0.3f * (float)replicas), c - 8) <= packed_ns;
+}
 
 __global__ void __launch_bounds__(kEnumThreads) k_sub_reduce(SubPrep* __restrict__ prep,
                                                              unsigned long long* keys)
@@ -550,7 +565,7 @@ __global__ void __launch_bounds__(kEnumThreads) k_sub_reduce(SubPrep* __restrict
         }
         if (lane == 0) {
             s_ncomp = nc;
-            s_solve = most <= 12 || most <= n - 4;
+            s_solve = enum_here(most, n, gridDim.x);
             s_S = 0;
         }
     }
