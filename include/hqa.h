@@ -104,7 +104,10 @@ enum {
     HQA_KERNEL_AUTO = 0,   /* vectorised when the blocking allows, else scalar */
     HQA_KERNEL_SCALAR = 1, /* one replica per lane, neighbour lists streamed from L1/L2 */
     HQA_KERNEL_VECTOR = 2, /* 16-byte gathers per lane, lists in shared memory; needs
-                              replicas_per_block >= 4 (FP32) or >= 8 (BF16) */
+                              replicas_per_block >= 4 (FP32) or >= 8 (BF16).  Half of
+                              that, which open options take for few replicas, is
+                              accepted as stated where hqa_autotune chose it for the
+                              context, replica count and precision */
     HQA_KERNEL_DENSE = 3,  /* dense contexts: the field as a GEMM of J and the replicas'
                               fluxes -- on the tcgen05 tensor cores for the 16-bit
                               precisions (BF16, BF16X2, FP16, FP16X2), on the CUDA cores
@@ -482,10 +485,11 @@ hqa_status hqa_hmd(hqa_ctx* ctx, const hqa_schedule* sched, double tau, int32_t 
 /* Autotuner: times each launch shape hqa_run can use for `replicas`
  * replicas at opts->precision (NULL = defaults) -- the scalar sparse kernel
  * at 1, 2, 4, ..., 32 replicas per block, the vectorised one at the
- * blockings that fill a 16-byte vector, the persistent batch kernels
- * (batch contexts: list-streaming at 1..32, HQA_KERNEL_LOWDEG at 1, 2, 4
- * when every member allows it), the dense tensor-core kernel (dense BF16/BF16X2)
- * -- on a probe anneal of probe_steps steps (1..100000; dt = 1/probe_steps,
+ * blockings that fill a 16-byte vector (and at half of that, or with both
+ * options left open for the complete-graph kernel, where open options take
+ * them), the streaming kernel, the persistent batch kernels (batch contexts:
+ * list-streaming at 1..32, HQA_KERNEL_LOWDEG at 1, 2, 4 when every member
+ * allows it), the dense kernels (dense contexts) -- on a probe anneal of probe_steps steps (1..100000; dt = 1/probe_steps,
  * init PAPER), one untimed run then three between CUDA events on `stream`.
  * The fastest is written to *best (the other fields from opts) and kept in
  * the context: later hqa_run calls for the same replica count and precision
@@ -497,8 +501,8 @@ hqa_status hqa_hmd(hqa_ctx* ctx, const hqa_schedule* sched, double tau, int32_t 
  * candidate runs, or called during a capture), OOM, CUDA, and a status a
  * probe latched (NONFINITE, TIMEOUT). */
 typedef struct {
-    int32_t kernel;               /* HQA_KERNEL_SCALAR, _VECTOR or _DENSE */
-    int32_t replicas_per_block;   /* 0 for the dense kernel */
+    int32_t kernel;               /* HQA_KERNEL_*; AUTO (with 0): open options */
+    int32_t replicas_per_block;   /* 0 for the dense and streaming kernels */
     double ms_per_step;           /* mean over the timed probes; -1 = rejected */
 } hqa_tune_entry;
 hqa_status hqa_autotune(hqa_ctx* ctx, const hqa_schedule* sched, int32_t replicas,

@@ -272,40 +272,58 @@ hqa_status check_opts(const hqa_run_opts& o)
     return HQA_OK;
 }
 
+// The blocking that an open call takes in the vectorised kernel where few replicas
+// would leave SMs idle: half of a 16-byte vector per lane where that still gives
+// every block an SM of its own, else 0.  A step's time is that of its block's
+// gathers, so idle SMs are worth more than wide loads: ER N = 800 x 300, 100
+// steps, FP32 381 -> 238 us, BF16 423 -> 269 us; N = 1000 of mean degree 8 x 256
+// 141 -> 99 and 197 -> 122 us.  Only where the blocking is left open or the
+// autotuner chose it; a stated one is taken as it is.
+int half_vector(const hqa_ctx* ctx, int32_t R, int prec)
+{
+    const int V = prec == HQA_PREC_BF16 ? 8 : 4;
+    const int rb = hqa_sparse_pick_rb(ctx, R, prec);
+    return rb > 0 && rb < V && R >= V && (R + V / 2 - 1) / (V / 2) <= ctx->sm_count &&
+                   hqa_vec_supported(ctx, V / 2, prec)
+               ? V / 2 : 0;
+}
+
+// Whether a run takes the complete-graph kernel: everything left open, and the
+// autotuner did not choose another one.
+bool takes_complete(const hqa_ctx* ctx, int32_t R, const hqa_run_opts& o)
+{
+    if (o.kernel != HQA_KERNEL_AUTO || o.replicas_per_block != 0 || !hqa_complete_possible(ctx, R))
+        return false;
+    const auto it = ctx->tuned.find({R, o.precision});
+    return it == ctx->tuned.end() || it->second.first == HQA_KERNEL_AUTO;
+}
+
 // Replica blocking and kernel variant: the vectorised kernel when the
 // blocking allows it and its shared-memory image fits, else the scalar one.
 hqa_status choose_plan(hqa_ctx* ctx, int32_t R, const hqa_run_opts& opts, const SparsePlan** plan)
 {
     if (opts.kernel == HQA_KERNEL_LOWDEG) return HQA_ERR_UNSUPPORTED;   // batch contexts only
     hqa_run_opts o = opts;
-    if (o.kernel == HQA_KERNEL_AUTO && o.replicas_per_block == 0) {
-        const auto it = ctx->tuned.find({R, o.precision});
-        if (it != ctx->tuned.end()) {
-            o.kernel = it->second.first;
-            o.replicas_per_block = it->second.second;
-        }
-    }
-    // A full 16-byte vector of replicas per lane, or half of one where that still
-    // gives every block an SM of its own.  A step's time is that of its block's
-    // gathers, so idle SMs are worth more than wide loads: ER N = 800 x 300, 100
-    // steps, FP32 381 -> 238 us, BF16 423 -> 269 us; N = 1000 of mean degree 8 x 256
-    // 141 -> 99 and 197 -> 122 us.  Only where the blocking is left open; a stated or
-    // tuned one is taken as it is.
     const int V = o.precision == HQA_PREC_BF16 ? 8 : 4;
-    const bool half_fits = R >= V && (R + V / 2 - 1) / (V / 2) <= ctx->sm_count &&
-                           hqa_vec_supported(ctx, V / 2, o.precision);
+    const auto it = ctx->tuned.find({R, o.precision});
+    if (o.kernel == HQA_KERNEL_AUTO && o.replicas_per_block == 0 && it != ctx->tuned.end()) {
+        o.kernel = it->second.first;
+        o.replicas_per_block = it->second.second;
+    }
     int RB = o.replicas_per_block;
     int rb_scalar = RB;   // the scalar kernel's blocking if the vectorised one is not used
-    bool narrow = false;
+    // half a vector: as the library's choice, or as the autotuner's for this run
+    bool narrow = o.kernel == HQA_KERNEL_VECTOR && RB == V / 2 && it != ctx->tuned.end() &&
+                  it->second == std::pair<int, int>(HQA_KERNEL_VECTOR, V / 2);
     if (RB == 0) {
         RB = rb_scalar = hqa_sparse_pick_rb(ctx, R, o.precision);
         if (o.kernel != HQA_KERNEL_SCALAR && RB < V && RB > 0 && R >= V) {
-            RB = V;
-            narrow = half_fits;
+            const int half = half_vector(ctx, R, o.precision);
+            RB = half ? half : V;
+            narrow = half != 0;
         }
     }
     if (RB == 0) return HQA_ERR_TOO_LARGE;
-    if (narrow) RB = V / 2;
     if (o.kernel != HQA_KERNEL_SCALAR && (narrow || RB >= V) && hqa_vec_supported(ctx, RB, o.precision)) {
         const SparsePlan* vp = nullptr;
         hqa_status s = hqa_vec_plan(ctx, RB, o.precision, &vp);
@@ -477,6 +495,8 @@ hqa_status run_batch(hqa_ctx* ctx, const hqa_schedule* sched, double dt, int64_t
 }
 
 }  // namespace
+
+int hqa_open_half_vector(const hqa_ctx* ctx, int32_t R, int prec) { return half_vector(ctx, R, prec); }
 
 extern "C" {
 
@@ -742,8 +762,7 @@ static hqa_status run_impl(hqa_ctx* ctx, const hqa_schedule* sched, double dt, i
         s = hqa_stream_launch_md(ctx, o.precision, ctx->d_sched, steps, sched->window, replicas,
                                  seed, o.init, o.phi0, o.p0, sched->M, out->phi, out->p, phibar,
                                  st);
-    else if (o.kernel == HQA_KERNEL_AUTO && o.replicas_per_block == 0 &&
-             hqa_complete_possible(ctx, replicas))
+    else if (takes_complete(ctx, replicas, o))
         s = hqa_complete_launch_md(ctx, o.precision, ctx->d_sched, steps, sched->window, replicas,
                                    seed, o.init, o.phi0, o.p0, sched->M, out->phi, out->p, phibar,
                                    st);
@@ -948,7 +967,7 @@ hqa_status hqa_plan_query(hqa_ctx* ctx, int32_t replicas, const hqa_run_opts* op
         out->balance = 1.0;
         return HQA_OK;
     }
-    if (o.kernel == HQA_KERNEL_AUTO && o.replicas_per_block == 0 && hqa_complete_possible(ctx, replicas)) {
+    if (takes_complete(ctx, replicas, o)) {
         out->kernel = HQA_KERNEL_SCALAR;
         out->replicas_per_block = 1;
         out->blocks = replicas;

@@ -298,6 +298,8 @@ hqa_status hqa_batch_launch_md(hqa_ctx* batch, int RB, int prec, const StepCoef*
                                const float* phi0, const float* p0, int M, float* phi_out,
                                float* p_out, float* phibar_out, cudaStream_t st);
 int hqa_sparse_pick_rb(const hqa_ctx* ctx, int32_t R, int prec);
+// api.cu: replicas per block of the half-vector form that an open call takes, or 0
+int hqa_open_half_vector(const hqa_ctx* ctx, int32_t R, int prec);
 // sparse_complete.cu: few replicas of a small complete graph
 bool hqa_complete_possible(const hqa_ctx* ctx, int32_t R);
 void hqa_complete_shape(const hqa_ctx* ctx, int32_t* threads, int64_t* smem_bytes);

@@ -5,14 +5,17 @@
 // Candidates: the scalar sparse kernel at 1..32 replicas per block, the
 // vectorised sparse kernel at the blockings that fill a 16-byte vector, the
 // persistent batch kernels (list-streaming at 1..32 replicas per block, the
-// low-degree one at 1, 2, 4 where every member allows it), and the dense
-// GEMM kernels (dense contexts: tcgen05 for the 16-bit precisions, the FP32
-// CUDA-core GEMM for FP32).  Each one
-// runs a short probe anneal (probe_steps leapfrog steps, dt = 1/probe_steps,
-// init PAPER) once untimed (plan build, caches) and then three times between
-// CUDA events on the caller's stream; the figure kept is the mean time per
-// step.  A candidate that the library rejects (shared memory, alignment of
-// the blocking, precision) is listed with ms_per_step = -1.
+// low-degree one at 1, 2, 4 where every member allows it), the streaming
+// kernel, and the dense GEMM kernels on the tensor cores (dense contexts).  What
+// an open call takes is always among them, so that a tuned context is not slower
+// than an untuned one: half a vector for few replicas (a candidate where an open
+// call takes it), and all options left open (0, 0) where that is the
+// complete-graph kernel, which no stated shape names.
+// Each candidate runs a short probe anneal (probe_steps leapfrog steps,
+// dt = 1/probe_steps, init PAPER) once untimed (plan build, caches) and then
+// three times between CUDA events on the caller's stream; the figure kept is
+// the mean time per step.  A candidate that the library rejects (shared memory,
+// alignment of the blocking, precision) is listed with ms_per_step = -1.
 #include <vector>
 
 #include "hqa_internal.cuh"
@@ -24,7 +27,7 @@ struct Cand {
     int rb;
 };
 
-std::vector<Cand> candidates(const hqa_ctx* ctx, int prec)
+std::vector<Cand> candidates(const hqa_ctx* ctx, int32_t R, int prec)
 {
     std::vector<Cand> c;
     const int rbs[6] = {1, 2, 4, 8, 16, 32};
@@ -32,8 +35,8 @@ std::vector<Cand> candidates(const hqa_ctx* ctx, int prec)
         c.push_back({HQA_KERNEL_DENSE, 0});
         return c;
     }
-    // FP32 on a dense context: the CUDA-core GEMM, and the sparse kernels
-    // when the couplings are all +-1
+    // FP32 on a dense context: the GEMM, and the sparse kernels when the
+    // couplings are all +-1
     if (prec == HQA_PREC_FP32 && hqa_simt_possible(ctx)) c.push_back({HQA_KERNEL_DENSE, 0});
     if (!ctx->unit || (prec != HQA_PREC_FP32 && prec != HQA_PREC_BF16)) return c;
     for (int rb : rbs) c.push_back({HQA_KERNEL_SCALAR, rb});
@@ -41,8 +44,10 @@ std::vector<Cand> candidates(const hqa_ctx* ctx, int prec)
         for (int rb : {1, 2, 4}) c.push_back({HQA_KERNEL_LOWDEG, rb});
     if (!ctx->is_batch) {
         const int V = prec == HQA_PREC_BF16 ? 8 : 4;
+        if (hqa_open_half_vector(ctx, R, prec)) c.push_back({HQA_KERNEL_VECTOR, V / 2});
         for (int rb : rbs)
             if (rb >= V) c.push_back({HQA_KERNEL_VECTOR, rb});
+        if (hqa_complete_possible(ctx, R)) c.push_back({HQA_KERNEL_AUTO, 0});
         if (hqa_stream_supported(ctx, prec)) c.push_back({HQA_KERNEL_STREAM, 0});
     }
     return c;
@@ -76,7 +81,7 @@ extern "C" hqa_status hqa_autotune(hqa_ctx* ctx, const hqa_schedule* sched, int3
     hqa_result res{};
     res.phi = static_cast<float*>(ctx->d_tune);
     res.p = res.phi + RN;
-    const std::vector<Cand> cands = candidates(ctx, o.precision);
+    const std::vector<Cand> cands = candidates(ctx, replicas, o.precision);
     cudaEvent_t e0, e1;
     HQA_CUDA_TRY(cudaEventCreate(&e0));
     if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -90,12 +95,12 @@ extern "C" hqa_status hqa_autotune(hqa_ctx* ctx, const hqa_schedule* sched, int3
     double best_ms = 0.0;
     std::vector<double> ms(cands.size(), -1.0);
     hqa_status fail = HQA_OK;
-    // the tuned table must not steer the probes themselves
-    auto saved = ctx->tuned.find({replicas, o.precision});
+    const auto saved = ctx->tuned.find({replicas, o.precision});
     const bool had = saved != ctx->tuned.end();
     const std::pair<int, int> old = had ? saved->second : std::pair<int, int>{0, 0};
-    ctx->tuned.erase({replicas, o.precision});
     for (size_t i = 0; i < cands.size() && fail == HQA_OK; ++i) {
+        // chosen while it is probed: half a vector is accepted only as the choice
+        ctx->tuned[{replicas, o.precision}] = {cands[i].kernel, cands[i].rb};
         hqa_run_opts c = o;
         c.kernel = cands[i].kernel;
         c.replicas_per_block = cands[i].rb;
@@ -133,6 +138,7 @@ extern "C" hqa_status hqa_autotune(hqa_ctx* ctx, const hqa_schedule* sched, int3
     }
     if (fail != HQA_OK || best_i < 0) {
         if (had) ctx->tuned[{replicas, o.precision}] = old;
+        else ctx->tuned.erase({replicas, o.precision});
         return fail != HQA_OK ? fail : HQA_ERR_UNSUPPORTED;
     }
     ctx->tuned[{replicas, o.precision}] = {cands[best_i].kernel, cands[best_i].rb};

@@ -1,0 +1,73 @@
+"""The autotuner knows what an open call takes: a tuned context is not slower than an untuned one."""
+import pytest
+
+from paper_2004_03972_gb300 import instances
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def hqa():
+    from paper_2004_03972_gb300 import hqa as h
+    return h
+
+
+def _ms(torch, run):
+    run()
+    best = 1e9
+    for _ in range(5):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        run()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("name,V", [("PREC_FP32", 4), ("PREC_BF16", 8)])
+def test_half_vector_is_a_candidate(hqa, name, V):
+    import torch
+    prec, R = getattr(hqa, name), 300
+    ctx = hqa.Context.from_instance(instances.er_pm1(800, 0.06, 1200))
+    before = ctx.plan(R, precision=prec)
+    assert (before["kernel"], before["replicas_per_block"]) == (hqa.KERNEL_VECTOR, V // 2)
+    half = dict(kernel=hqa.KERNEL_VECTOR, replicas_per_block=V // 2, precision=prec)
+    with pytest.raises(hqa.HQAError):           # a choice of the library's, not of the caller's
+        ctx.plan(R, **half)
+    kw = dict(seed=4, dt=1e-3, precision=prec, outputs=("phi", "p"))
+    untuned = _ms(torch, lambda: ctx.run(100, R, **kw))
+    best, rows = ctx.autotune(R, precision=prec, probe_steps=100)
+    assert any(r[:2] == (hqa.KERNEL_VECTOR, V // 2) and r[2] > 0 for r in rows)
+    assert (best["kernel"], best["replicas_per_block"]) == min((r for r in rows if r[2] > 0), key=lambda r: r[2])[:2]
+    # the margin is for the clock: the full vector takes 1.57 times as long
+    assert _ms(torch, lambda: ctx.run(100, R, **kw)) <= 1.15 * untuned
+    a = ctx.run(100, R, **kw)
+    b = ctx.run(100, R, kernel=best["kernel"], replicas_per_block=best["replicas_per_block"], **kw)
+    ctx.sync()
+    assert all(torch.equal(a[k], b[k]) for k in a)
+    if best["replicas_per_block"] == V // 2:
+        for R2, p2 in ((R - 4, prec), (R, 1 - prec)):
+            with pytest.raises(hqa.HQAError):
+                ctx.plan(R2, **dict(half, precision=p2, replicas_per_block=2 if p2 == 0 else 4))
+    ctx.close()
+
+
+@pytest.mark.parametrize("N,R", [(100, 1), (256, 40)])
+def test_complete_graph_stays_open(hqa, N, R):
+    import torch
+    ctx = hqa.Context.from_instance(instances.sk_pm1(N, 2))
+    before = ctx.plan(R)
+    kw = dict(seed=4, dt=1e-3, outputs=("phi", "p"))
+    untuned = _ms(torch, lambda: ctx.run(200, R, **kw))
+    best, rows = ctx.autotune(R, probe_steps=100)
+    assert (hqa.KERNEL_AUTO, 0) in [r[:2] for r in rows]
+    assert (best["kernel"], best["replicas_per_block"]) == (hqa.KERNEL_AUTO, 0)   # three times faster
+    assert ctx.plan(R) == before
+    assert _ms(torch, lambda: ctx.run(200, R, **kw)) <= 1.15 * untuned
+    a = ctx.run(50, R, **kw)
+    b = ctx.run(50, R, kernel=best["kernel"], replicas_per_block=best["replicas_per_block"], **kw)
+    ctx.sync()
+    assert all(torch.equal(a[k], b[k]) for k in a)
+    ctx.close()
+
