@@ -489,7 +489,8 @@ hqa_status hqa_hmd(hqa_ctx* ctx, const hqa_schedule* sched, double tau, int32_t 
  * options left open for the complete-graph kernel, where open options take
  * them), the streaming kernel, the persistent batch kernels (batch contexts:
  * list-streaming at 1..32, HQA_KERNEL_LOWDEG at 1, 2, 4 when every member
- * allows it), the dense kernels (dense contexts) -- on a probe anneal of probe_steps steps (1..100000; dt = 1/probe_steps,
+ * allows it, timed as a call with open options then runs it: small members take
+ * more replicas per work item), the dense kernels (dense contexts) -- on a probe anneal of probe_steps steps (1..100000; dt = 1/probe_steps,
  * init PAPER), one untimed run then three between CUDA events on `stream`.
  * The fastest is written to *best (the other fields from opts) and kept in
  * the context: later hqa_run calls for the same replica count and precision

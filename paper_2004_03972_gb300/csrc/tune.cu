@@ -10,7 +10,8 @@
 // an open call takes is always among them, so that a tuned context is not slower
 // than an untuned one: half a vector for few replicas (a candidate where an open
 // call takes it), and all options left open (0, 0) where that is the
-// complete-graph kernel, which no stated shape names.
+// complete-graph kernel, which no stated shape names.  A low-degree blocking is
+// timed as a tuned open call runs it, with larger items for small members.
 // Each candidate runs a short probe anneal (probe_steps leapfrog steps,
 // dt = 1/probe_steps, init PAPER) once untimed (plan build, caches) and then
 // three times between CUDA events on the caller's stream; the figure kept is
@@ -99,11 +100,13 @@ extern "C" hqa_status hqa_autotune(hqa_ctx* ctx, const hqa_schedule* sched, int3
     const bool had = saved != ctx->tuned.end();
     const std::pair<int, int> old = had ? saved->second : std::pair<int, int>{0, 0};
     for (size_t i = 0; i < cands.size() && fail == HQA_OK; ++i) {
-        // chosen while it is probed: half a vector is accepted only as the choice
+        // chosen while it is probed: half a vector is accepted only as the choice,
+        // and a low-degree blocking left open is the one that the choice stands for
         ctx->tuned[{replicas, o.precision}] = {cands[i].kernel, cands[i].rb};
         hqa_run_opts c = o;
-        c.kernel = cands[i].kernel;
-        c.replicas_per_block = cands[i].rb;
+        const bool open = cands[i].kernel == HQA_KERNEL_LOWDEG;
+        c.kernel = open ? HQA_KERNEL_AUTO : cands[i].kernel;
+        c.replicas_per_block = open ? 0 : cands[i].rb;
         s = hqa_run(ctx, sched, dt, probe_steps, replicas, 0, &c, &res, stream);
         if (s == HQA_ERR_CUDA || s == HQA_ERR_OOM) fail = s;
         if (s != HQA_OK) continue;
