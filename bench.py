@@ -5,12 +5,13 @@ With no --config, the line's headline is the largest single-GPU workload, the
 paper's MAX-CUT shape (Results, "HQA for MAX-CUT"; Methods, "MAX-CUT and Ising
 spin-glass"): SK / K2000 with +-1 weights, 4096 replicas, 10000 leapfrog steps
 of the paper's schedule.  The same JSON line carries, under "nested", the
-sparse ER workload and the uneven batch, each with its own roofline, CPU
-baseline and end-to-end figure.
+rate, end-to-end rate and roofline fraction of the sparse ER workload, the
+uneven batch and the surrogate-gated runs; --detail FILE writes the full
+record.
 
 Workloads (--config):
   sk2000  K2000 +-1 dense, 4096 replicas, 10000 steps, dense GEMM field.
-          Variants: plain FP32 (CUDA-core GEMM, the reference form), FP16X2
+          Variants: plain FP32 (tcgen05, phi in three exact BF16 slices), FP16X2
           (tcgen05, phi split into two FP16 halves, ~22 significant bits),
           FP16 and BF16 (tcgen05, one 16-bit operand; stated errors).
   er800   Erdos-Renyi G(800, 0.06) +-1 CSR, 1024 replicas, 5000 steps, under
@@ -29,7 +30,7 @@ Spin-updates per step = N * R * S (one leapfrog step of one spin in one replica)
 The headline variant is the fastest whose 100-step state parity meets the
 contract (1e-2 of the FP64 oracle for low precision) and whose median cut is
 not worse than the plain FP32 variant's (the 95% bootstrap interval of the
-median difference reaches 0); every variant is reported under "variants".
+median difference reaches 0); every variant's rate stands under "variants".
 
 The reference arm (--impl reference) times the FP64 CPU oracle on the host
 cores over a bounded sample of the same workload (the paper has no code).
@@ -440,8 +441,8 @@ def measure(name, args, hqa, torch, timer, dev, ws, rank, headline):
             tuned = {"kernel": best["kernel"], "replicas_per_block": best["replicas_per_block"],
                      "candidates": [[k, rb, round(ms, 6)] for k, rb, ms in rows]}
         slow = prec_name == "PREC_FP32" and (kern_name == "KERNEL_DENSE" or v["one_at_a_time"])
-        # the plain dense FP32 form and the one-at-a-time baseline take a few seconds a
-        # step: two timed steps; variants outside the parity contract: five
+        # the plain dense FP32 form and the one-at-a-time baseline take longest: two
+        # timed steps; variants outside the parity contract: five
         Kv = min(K, 2) if slow else (K if cfg["parity"][vname][1] else min(K, 5))
         quality = []
 
@@ -617,6 +618,8 @@ def measure(name, args, hqa, torch, timer, dev, ws, rank, headline):
                 "median_energy_gain_over_readout": float(gain.median())}
     cpu = cpu_baseline(args, inst, cfg) if (rank == 0 and not args.skip_cpu) else None
     launches = launches_per_step(hqa, plan, hv, cfg, S, batch, real, count)
+    if not (batch or real or hv["one_at_a_time"]):
+        launches += 1         # the sub-solve's reduction
     rec = {
         "value": value, "unit": "spin-updates/s", "steps": hv["steps"],
         "warmup": W, "ms_per_step": 1e3 * tot_pipe / hv["steps"],
@@ -882,6 +885,43 @@ def cpu_baseline(args, inst, cfg):
                       "(MD only, FP64, OpenMP over replicas)"}
 
 
+# Keys of the printed line.  It has to survive a reader that keeps the last few kilobytes of the
+# output, so it holds the figures and leaves tables (autotuner candidates, plans, cut intervals,
+# gated points) to the full record (--detail).
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+             "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "gpu_launches",
+             "config", "e2e", "clocks", "headline_variant")
+ROOF_KEYS = ("bound", "achieved", "peak", "unit", "frac", "issued_tflops", "issued_frac", "kernel",
+             "launch_ms", "traffic")
+
+
+def _short(x):
+    """Floats to six significant digits, all the way down."""
+    if isinstance(x, dict):
+        return {k: _short(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [_short(v) for v in x]
+    return float(f"{x:.6g}") if isinstance(x, float) else x
+
+
+def printed_line(rec):
+    """The one line of a full record."""
+    line = {k: rec[k] for k in LINE_KEYS if k in rec}
+    roof = rec.get("roofline") or {}
+    line["roofline"] = {k: roof[k] for k in ROOF_KEYS if k in roof}
+    if rec.get("cpu_baseline"):
+        line["cpu_baseline"] = rec["cpu_baseline"]
+    if "variants" in rec:
+        line["variants"] = {k: v["spin_updates_per_s"] for k, v in rec["variants"].items()}
+    if "nested" in rec:
+        line["nested"] = {k: {"value": v["value"], "unit": v["unit"],
+                              "e2e": (v.get("e2e") or {}).get("value"),
+                              "roofline_frac": (v.get("roofline") or {}).get("frac"),
+                              "kernel": (v.get("roofline") or {}).get("kernel")}
+                          for k, v in rec["nested"].items()}
+    return _short(line)
+
+
 def run_ours(args):
     import torch
 
@@ -923,7 +963,10 @@ def run_ours(args):
     if sub:
         line["nested"] = sub
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(printed_line(line)), flush=True)
     if ws > 1:
         torch.distributed.destroy_process_group()
 
@@ -969,6 +1012,8 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--config", default="all", choices=["all", "er_surrogate"] + sorted(CONFIGS))
     ap.add_argument("--skip-cpu", action="store_true")
+    ap.add_argument("--detail", default="", metavar="FILE",
+                    help="also write the full record (every variant, candidate and interval) there")
     ap.add_argument("--md-steps", type=int, default=0,
                     help="override the workload's MD step count (shorter runs for profiling)")
     ap.add_argument("--no-tune", action="store_true",
