@@ -323,13 +323,15 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
         int i = i0, v = v0;
         for (int l = threadIdx.x; l < mine; l += kMDThreads) {
             const int c = v * V;
+            const size_t o = (size_t)i * a.Rpad + c;
+            float own[V];   // FP32: the cell's own flux, on its way with the gathers
+            if constexpr (!BF16) Vec<false>::load(cur, o, own);
             float L[V];
             if constexpr (STAGED)
                 row_sum<BF16>(cur, a.Rpad, c, s_off[i - rowA], s_off[i - rowA + 1],
                               [&](int k) { return s_ent[k]; }, L);
             else
                 cell_field<BF16>(a, cur, i, c, L);
-            const size_t o = (size_t)i * a.Rpad + c;
             const float hr = a.h ? 2.f * __ldg(a.h + i) : 0.f;
             const bool res = l < nres;
             float sv[4 * NP], fn[V];
@@ -337,11 +339,7 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
             for (int q = 0; q < NP; ++q) get4(sv + 4 * q, res ? st + q * a.nres + l : gplane(q, o));
             float* ph = sv;
             float* pp = sv + (BF16 ? 8 : 0);
-            float own[V];
-            if constexpr (!BF16) {
-                Vec<false>::load(cur, o, own);
-                ph = own;
-            }
+            if constexpr (!BF16) ph = own;
 #pragma unroll
             for (int e = 0; e < V; ++e) {
                 const float Le = hr != 0.f ? L[e] + hr * fabsf(ph[e]) : L[e];
