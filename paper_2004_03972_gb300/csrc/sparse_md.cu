@@ -254,14 +254,17 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sparse_md(const MDArgs a)
 
 // One replica per CTA on a small instance (a few tuples), where a step is a
 // chain of latencies: the kernel above leaves it to one warp per tuple, which
-// walks its list alone (SK N = 100: four warps, 1.4 us per step).  Here all 32
-// warps take the tuples' list chunks (four gathers and their sum, the first
-// kHeld chunks' offsets in registers), the sums pass through shared memory, and
-// a row's owner adds them up in the order of the list.  Same operations in the
-// same order as md_block, so the same bits.  Flux, momentum and window sum stay
-// in the owner's registers.  SK N = 100, one replica: 1.40 -> 0.88 us per
-// step; half of it is the gathers' shared-memory wavefronts (480 and 300 of bank
-// conflicts), the rest the owners' sums and two barriers.
+// walks its list alone.  Here up to 32 warps share the tuples' list chunks (four
+// gathers and their sum, the first kHeld chunks' offsets in registers), the sums
+// pass through shared memory, and a row's owner adds them up in the order of the
+// list.  Same operations in the same order as md_block, so the same bits.  Flux,
+// momentum and window sum stay in the owner's registers.  As many warps as have
+// kHeld chunks each: more only lengthen the two barriers.  One replica, us per
+// step, a warp per tuple / a warp per chunk / a warp per four: mean degree 8,
+// N = 250 0.65 / 0.75 / 0.49; density 0.2, N = 100 0.75 / 0.69 / 0.43, N = 160
+// 0.92 / 0.79 / 0.56, N = 256 1.29 / 1.22 / 1.22; density 0.97, N = 128 1.60 / 1.15 /
+// 1.16, N = 200 2.57 / 2.67 / 2.67, the one size found that loses.  What is left
+// are the gathers' shared-memory wavefronts, the owners' sums and two barriers.
 constexpr int kHeld = 4;
 constexpr int kSplitTuples = 8;
 constexpr uint32_t kSplitBuf = 2048;   // bytes per operand buffer: a constant, so that the
@@ -735,7 +738,7 @@ hqa_status hqa_sparse_launch_md(hqa_ctx* ctx, const SparsePlan* pl, const StepCo
         const void* fn = bf ? (const void*)k_sparse_md_split<true> : (const void*)k_sparse_md_split<false>;
         if (hqa_smem_attr(fn, split) != cudaSuccess) return HQA_ERR_CUDA;
         int chunks = (int)pl->chunks;
-        const int warps = std::max(pl->T, std::min(32, chunks));
+        const int warps = std::max(pl->T, std::min(32, (chunks + kHeld - 1) / kHeld));
         void* args[] = {&a, &chunks};
         return cudaLaunchKernel(fn, dim3(R), dim3(32 * warps), args, split, st) == cudaSuccess
                    ? HQA_OK : HQA_ERR_CUDA;
