@@ -321,7 +321,13 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
         void* nxt = (m & 1) ? a.op0 : a.op1;
         const bool in_win = m >= win0;
         int i = i0, v = v0;
-        for (int l = threadIdx.x; l < mine; l += kMDThreads) {
+        // FP32: all lanes of a warp take part in every round, see below
+        for (int l = threadIdx.x; (BF16 ? l : l - (int)threadIdx.x) < mine; l += kMDThreads) {
+            const bool on = BF16 || l < mine;
+            if (!on) {
+                i = rowA;
+                v = 0;
+            }
             const int c = v * V;
             const size_t o = (size_t)i * a.Rpad + c;
             float own[V];   // FP32: the cell's own flux, on its way with the gathers
@@ -332,6 +338,12 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
                               [&](int k) { return s_ent[k]; }, L);
             else
                 cell_field<BF16>(a, cur, i, c, L);
+            // Where a warp's lanes lie in two rows or more, their sums end at different
+            // passes, and without this they stay apart up to the barrier: FP32, N =
+            // 40000 x 100 21.9 -> 16.1 us a step, 20000 x 200 16.2 -> 15.2.  In BF16 the
+            // same cost 3 %.
+            if constexpr (!BF16) __syncwarp();
+            if (!on) break;
             const float hr = a.h ? 2.f * __ldg(a.h + i) : 0.f;
             const bool res = l < nres;
             float sv[4 * NP], fn[V];

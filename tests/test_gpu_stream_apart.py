@@ -1,0 +1,55 @@
+"""FP32 streaming rows that are no multiple of a warp: the lanes of a warp come together again
+after their sums (40000 spins x 100 replicas: 16 us a step, 22 while they stayed apart)."""
+import pytest
+
+from paper_2004_03972_gb300 import instances
+
+pytestmark = pytest.mark.gpu
+
+
+def _step_us(torch, hqa, ctx, R):
+    out = {k: torch.empty(R, ctx.N, device="cuda") for k in ("phi", "p")}
+    ms = {}
+    for S in (50, 250):
+        run = lambda: ctx.run(S, R, seed=1, dt=1e-4, sched=hqa.schedule(window=1),
+                              kernel=hqa.KERNEL_STREAM, out=out)
+        run()
+        ms[S] = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            run()
+            b.record()
+            torch.cuda.synchronize()
+            ms[S] = min(ms[S], a.elapsed_time(b))
+    return (ms[250] - ms[50]) / 200 * 1e3
+
+
+def test_odd_rows_are_not_slower_than_longer_ones():
+    """25 vectors a row against 32: less to move, and no more time."""
+    import torch
+
+    from paper_2004_03972_gb300 import hqa
+    ctx = hqa.Context.from_instance(instances.er_mean_degree_pm1(40000, 8, 1))
+    odd, even = _step_us(torch, hqa, ctx, 100), _step_us(torch, hqa, ctx, 128)
+    assert odd <= 1.1 * even
+    ctx.close()
+
+
+@pytest.mark.parametrize("R", [97, 100, 180, 300])
+def test_same_bits_as_resident(R):
+    """Whole-number fluxes: every sum is exact, so one step equals the list kernel's."""
+    import torch
+
+    from paper_2004_03972_gb300 import hqa
+    N = 1500
+    ctx = hqa.Context.from_instance(instances.er_mean_degree_pm1(N, 8, 2))
+    g = torch.Generator("cuda").manual_seed(R)
+    phi = torch.randint(-8, 9, (R, N), generator=g, device="cuda").float()
+    p0 = torch.rand(R, N, generator=g, device="cuda") - 0.5
+    kw = dict(dt=1e-3, init=hqa.INIT_GIVEN, phi0=phi, p0=p0, start_step=100, outputs=("phi", "p", "phibar"))
+    a = ctx.run(1, R, kernel=hqa.KERNEL_STREAM, **kw)
+    b = ctx.run(1, R, kernel=hqa.KERNEL_SCALAR, replicas_per_block=1, **kw)
+    ctx.sync()
+    assert all(torch.equal(a[k], b[k]) for k in a)
+    ctx.close()
