@@ -27,8 +27,9 @@
 // step moved through L2 at N = 20000 x 256 in BF16, and one CTA per SM makes a
 // barrier 152 arrivals instead of one per 256 threads.  Per step there: BF16
 // 20.9 -> 14.7 us, FP32 20.6 -> 19.4 us, and with the ranges cut at whole warps
-// (first_cell) 12.2 and 16.0; N = 8000 x 40 FP32 5.4 -> 4.1 us, mostly the barrier
-// and two rounds of gathers.
+// (first_cell) 12.4 and 17.2; N = 8000 x 40 FP32 5.3 -> 3.9 us, mostly the barrier
+// and two rounds of gathers.  Beyond L2 (operand buffers, sums and the state that is
+// not resident above about 100 MB) this form and the one before it are within 7 %.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -266,7 +267,8 @@ __device__ __forceinline__ void get4(float* x, const float4* src)
 // First cell of CTA b of g, in units of 32 where rows are a multiple of 32 vectors:
 // a warp then stays within one row (one list length, four full lines per gather).
 // N = 20000 x 256 BF16, 100 steps, 1888 -> 1637 us, FP32, 60 steps, 1454 -> 1250 us;
-// other row lengths, where a warp spans rows all the same, lost up to 9 %.
+// other row lengths, where a warp spans rows all the same, lost up to 9 % (measured
+// before the lanes of a warp met after their sums).
 __host__ __device__ inline int64_t cell_unit(int nv) { return nv % 32 == 0 ? 32 : 1; }
 __host__ __device__ inline int64_t first_cell(int64_t cells, int nv, int64_t b, int64_t g)
 {
@@ -617,14 +619,25 @@ hqa_status hqa_stream_launch_md(hqa_ctx* ctx, int prec, const StepCoef* d_sched,
     const int64_t most = (cells / cell_unit(nv) + grid - 1) / grid * cell_unit(nv);   // of a CTA
     a.nres = (int)std::min<int64_t>(most,
                                     (int64_t)((ctx->smem_optin - 1024 - lists) / cell_bytes));
+    const size_t n = (size_t)ctx->N * a.Rpad;
+    // bytes of operand buffers and state in global memory, with nres cells a CTA resident
+    const auto touched = [&](int nres) {
+        const double spilled = std::max(0.0, 1.0 - (double)nres * grid / (double)cells);
+        return (double)n * (2 * (bf16 ? 2 : 4) + spilled * (bf16 ? 8 : 4));
+    };
+    // Beyond L2 gathers wait for DRAM, and what holds them meanwhile is L1, which
+    // shares its memory with the resident state: rows that spread over more lines
+    // (no whole warps) then gain more from L1.  us per step, all that fits resident /
+    // this many: FP32 N = 60000 x 300 109 / 91, 60000 x 240 76 / 68; BF16 60000 x 400
+    // 122 / 103, 40000 x 400 70 / 65; rows of whole warps lost 5 %.
+    if (nv % 32 != 0 && touched(a.nres) > 0.8 * (double)ctx->l2_bytes)
+        a.nres = std::min(a.nres, bf16 ? 1024 : 6144);
     const size_t smem = a.nres * cell_bytes + lists;
     // window sums by reductions while what a step touches in global memory (both
     // operand buffers, the sums, the state that is not resident) stays in L2;
     // beyond, a reduction waits for its line from DRAM in L2 and holds up the
     // gathers (N = 40000 x 256 BF16, 100 steps: 5.5 ms without, 5.9 with)
-    const size_t n = (size_t)ctx->N * a.Rpad;
-    const double spilled = std::max(0.0, 1.0 - (double)a.nres * grid / (double)cells);
-    a.wred = (double)n * (2 * (bf16 ? 2 : 4) + 4 + spilled * (bf16 ? 8 : 4)) < 0.7 * (double)ctx->l2_bytes;
+    a.wred = touched(a.nres) + 4.0 * (double)n < 0.7 * (double)ctx->l2_bytes;
     const void* fn = bf16 ? (staged ? (const void*)k_sparse_stream<true, true>
                                     : (const void*)k_sparse_stream<true, false>)
                           : (staged ? (const void*)k_sparse_stream<false, true>

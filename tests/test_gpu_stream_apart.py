@@ -36,6 +36,18 @@ def test_odd_rows_are_not_slower_than_longer_ones():
     ctx.close()
 
 
+def test_sets_beyond_l2():
+    """N = 60000 x 300 moves 300 / 256 of what x 256 does: 1.18 times its time for that, 1.4 while
+    the resident state left L1 too small for gathers that wait for DRAM."""
+    import torch
+
+    from paper_2004_03972_gb300 import hqa
+    ctx = hqa.Context.from_instance(instances.er_mean_degree_pm1(60000, 8, 1))
+    odd, even = _step_us(torch, hqa, ctx, 300), _step_us(torch, hqa, ctx, 256)
+    assert odd / 300 <= 1.3 * even / 256
+    ctx.close()
+
+
 @pytest.mark.parametrize("R", [97, 100, 180, 300])
 def test_same_bits_as_resident(R):
     """Whole-number fluxes: every sum is exact, so one step equals the list kernel's."""
