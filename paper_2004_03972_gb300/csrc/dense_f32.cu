@@ -2,8 +2,8 @@
 //
 // The field L = J Phi of an FP32 run (Methods, "Leapfrog algorithm") is a
 // contraction that the CUDA cores bound at 80 TFLOP/s.  Here it runs on the
-// BF16 tensor cores from fixed-point slices, at an error against FP64 that is
-// below the FP32 sum's:
+// BF16 tensor cores from slices of phi, at an error against FP64 that is below
+// the FP32 sum's in all but the states named below:
 //
 //   phi = b0 + b1 + b2,  b0 = phi rounded to a multiple of u, then to BF16,
 //                        b1 = the rest rounded to BF16,
@@ -25,10 +25,17 @@
 // has the bits of an unbroken one, and the accuracy is the same at every scale of
 // phi.  One unit for 16 to 64 replicas, taken from the largest |phi| two steps
 // before, cost a replica 1000 times smaller than its neighbours two digits.
-// Where the 32-spin groups of one replica differ in scale by 2^10 and more, the
-// small groups' b0 is truncated against the sum of the large ones: there the error
-// is up to 2.6 times the FP32 sum's (a restatement in 64 bits, N = 2000), elsewhere
-// a tenth of it or less.
+//
+// Error of the field against FP64 (2-norm over a replica's spins, the largest of
+// 40), these slices / the FP32 sum on the CUDA cores: uniform, normal and
+// log-uniform fluxes at any scale 2.6e-8 to 7e-8 / 1.9e-7 at N = 64, 2.6e-8
+// (+-1) and 1.5e-7 (real) / 8.5e-7 at 2000, 3e-7 / 2.0e-6 at 12000.  Where the
+// 32-spin groups of ONE replica differ in scale by 2^6 (real J, large N) to 2^10
+// (+-1), the small groups' b0 is truncated against the sum of the large ones, up
+// to half a last place per 16 spins: every other 64 spins 1e-5 of the rest
+// 1.4e-6 / 8.6e-7 at N = 2000 and 7.4e-6 / 2.0e-6 at 12000, one flux 2^20 times
+// all others 4.5e-6 / 1.3e-6 and 2.5e-5 / 3e-6.  A unit for the whole replica would
+// mend that and take bits from small groups that couple among themselves only.
 //
 // Couplings: +-1 (any integer up to 127) is one exact BF16 slice.  Real
 // couplings are cut the same way (a_0 + a_1 + a_2; a_0 a multiple of 2^-7 of a
@@ -44,15 +51,19 @@
 // pairs of row tiles share cta_group::2 MMAs where the row tiles pair up and
 // J is one slice.  While the producer waits for the column group it already
 // loads coupling tiles into free stages, since only phi depends on the other
-// CTAs (real N = 500 x 200: 7.3 -> 6.9 us per step; filling the ring before
-// looking at the counter cost K2000 x 1024 17.5 -> 18.5 us).
+// CTAs (real N = 500 x 200: 7.3 -> 6.9 us per step, measured with that unit, as
+// is the next; filling the ring before looking at the counter cost K2000 x 1024
+// 17.5 -> 18.5 us).
 //
 // What bounds it: the SM's intake from L2, 28 KB per k-tile of a pair's CTA at
 // about 100 GB/s of the 128 that an SM can take (64 B/clk); the MMAs would need
-// two thirds of the step.  Measured against the CUDA-core form
-// (dense_simt.cu), per step: K2000 +-1 x 1024 replicas 210 -> 17.5 us, real
-// N = 1000 x 512 115 -> 10.6 us; error against FP64 after 40 steps (2-norm, p)
-// 6.9e-7 -> 3.8e-7 and 7.6e-7 -> 4.9e-7.
+// two thirds of the step.  Real couplings of N = 1000 x 512 the same: 60 KB per
+// k-tile (three coupling slices), 960 KB a step at 90 GB/s.  Measured against the
+// CUDA-core form (dense_simt.cu), per step: K2000 +-1 x 1024 replicas 210 -> 16.5
+// us, real N = 1000 x 512 115 -> 10.7 us; error against FP64 after 40 steps (2-norm,
+// p) 6.9e-7 -> 3.7e-7 and 7.6e-7 -> 4.7e-7.  (A unit from the largest |phi| of the
+// replicas that share a tile, passed between the CTAs each step, took 17.5 and
+// 12.0 us.)
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -150,6 +161,7 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                    done_bar = accf0 + 40;
     static_assert(24 * STAGES + 48 <= 1024, "barrier block");
     __shared__ int s_abort;
+    __shared__ uint32_t s_tiny;   // *a.tiny: here, as a register held through the steps costs up to 3 %
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mt = blockIdx.x % a.Mt, nc = blockIdx.x / a.Mt;
     const uint32_t crank = PAIR ? tc::cluster_rank() : 0u;
@@ -157,6 +169,7 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
 
     if (threadIdx.x == 0) {
         s_abort = 0;
+        s_tiny = __ldcg(a.tiny);
         for (int s = 0; s < STAGES; ++s) {
             tc::mbar_init(full0 + 8 * s, 1);
             tc::mbar_init(empty0 + 8 * s, 1);
@@ -352,7 +365,6 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
         const float rs = a.rscale ? a.rscale[row] : 1.f;
         const int mhalf = (a.M - 2) / 2;
         const int64_t win0 = a.S - (int64_t)a.W;
-        const bool tiny = __ldcg(a.tiny) != 0u;
         const uint32_t tl = tmem + ((uint32_t)(32 * quarter) << 16);
         const uint32_t rloc = (uint32_t)(32 * quarter + lane);
         const uint32_t acce_to = (PAIR && crank != 0) ? tc::mapa(acce0, 0) : acce0;
@@ -371,7 +383,7 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
         bool stop = false;
         for (int64_t m = 0; m < a.S && !stop; ++m) {
             const float4 cf = __ldg(reinterpret_cast<const float4*>(a.sched) + m);
-            const bool in_win = m >= win0 && !tiny, plain_win = m >= win0 && tiny;
+            const bool in_win = m >= win0 && *(volatile uint32_t*)&s_tiny == 0u;
             for (int hh = 0; hh < HV && !stop; ++hh) {
                 float pp[16];
                 if (row_ok && csel < NC / 16) {
@@ -436,12 +448,6 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                                     win_add(a.w + o1, fh);
                                 }
                             }
-                            if (plain_win) {
-                                float f[16];
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(fv[j]);
-                                hqa_win_plain16(a.w + (size_t)(n0 + col) * a.Npad + row, a.Npad, f);
-                            }
                         }
                         // the operand; spin rows beyond N keep a zero one
 #pragma unroll
@@ -459,6 +465,9 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                         // .sync.aligned: every lane of the warp, outside the row_ok branch
                         tc::tmem_st16(tl + PHI0 + (uint32_t)col, fv);
                         tc::tmem_wait_st();
+                        if (m >= win0 && !in_win)
+                            win_plain_tmem(a.w + (size_t)(n0 + col) * a.Npad + row, a.Npad,
+                                           tl + PHI0 + (uint32_t)col, row_ok);
                         tc::fence_proxy_async_smem();
                         tc::named_bar(2 + csel, 128);
                         if (gleader) {
@@ -777,7 +786,7 @@ static int unit_steps(double sum, bool whole)
 }
 
 // Coupling slices, built on first use: the BF16 copy of J when J is whole
-// numbers up to 127, else up to three fixed-point slices per row.
+// numbers up to 127, else up to three slices per row.
 hqa_status hqa_f32tc_prepare(hqa_ctx* ctx)
 {
     if (ctx->f32_nj) return HQA_OK;

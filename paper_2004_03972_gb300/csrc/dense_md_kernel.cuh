@@ -88,6 +88,26 @@ constexpr uint32_t kStgBytes = 16 * 128 * 2;   // one staging tile [16 replicas]
 // outside the window a step is unchanged (43 and 30 us).
 __device__ __forceinline__ void win_add(float* w, float v) { atomicAdd(w, v); }
 
+// The same by load, add and store, for marked states: volatile, so past L1 and one
+// after another.  The fluxes are read back from where the step left them, so that
+// the update holds no register for it.
+__device__ __forceinline__ void win_plain(float* w, float v)
+{
+    volatile float* o = w;
+    *o = *o + v;
+}
+
+__device__ __forceinline__ void win_plain_tmem(float* w, size_t stride, uint32_t taddr, bool row_ok)
+{
+    uint32_t v[16];
+    tc::tmem_ld16(taddr, v);   // .sync.aligned: every lane of the warp
+    tc::tmem_wait_ld();
+    if (row_ok) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) win_plain(w + j * stride, __uint_as_float(v[j]));
+    }
+}
+
 __device__ __forceinline__ void sts_u16(uint32_t a, uint16_t v)
 {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(v) : "memory");
@@ -217,6 +237,7 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
     // shared memory left to the ring
     const uint32_t phis = bar + 1024;
     __shared__ int s_abort;
+    __shared__ uint32_t s_tiny;   // *a.tiny: here, as a register held through the steps costs up to 3 %
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mt = blockIdx.x % a.Mt, nc = blockIdx.x / a.Mt;
     // PAIR: rank 0 (the even row tile) issues the MMAs; clusters are consecutive CTAs
@@ -225,6 +246,7 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
 
     if (threadIdx.x == 0) {
         s_abort = 0;
+        s_tiny = __ldcg(a.tiny);
         for (int s = 0; s < STAGES; ++s) {
             tc::mbar_init(full0 + 8 * s, 1);
             tc::mbar_init(empty0 + 8 * s, 1);
@@ -432,7 +454,6 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
         const float hr = (a.h && row_ok) ? 2.f * a.h[row] : 0.f;
         const int mhalf = (a.M - 2) / 2;
         const int64_t win0 = a.S - (int64_t)a.W;
-        const bool tiny = __ldcg(a.tiny) != 0u;
         const uint32_t tl = (uint32_t)(32 * quarter) << 16;   // this warp's TMEM lanes
         const uint32_t rloc = (uint32_t)(32 * quarter + lane);  // row within the tile
         // PAIR, odd CTA: accumulators are released on the even CTA's barrier
@@ -466,7 +487,7 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
         bool stop = false;
         for (int64_t m = 0; m < a.S && !stop; ++m) {
             const float4 cf = __ldg(reinterpret_cast<const float4*>(a.sched) + m);
-            const bool in_win = m >= win0 && !tiny, plain_win = m >= win0 && tiny;
+            const bool in_win = m >= win0 && *(volatile uint32_t*)&s_tiny == 0u;
             const int Kb = KSEG * a.Npad;   // operand row: [hi], [hi | lo] or [hi | hi | lo]
             uint16_t* nb = a.phib + (size_t)((m + 1) & 1) * a.Rpad * Kb;
             bool ok = true;
@@ -594,15 +615,12 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
                                 if constexpr (KSEG != 1) sts_u16(sb + kStgBytes, 0);
                             }
                         }
-                        if (plain_win && row_ok) {
-                            float f[16];
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(fv[j]);
-                            hqa_win_plain16(a.w + (size_t)(n0 + col) * a.Npad + row, a.Npad, f);
-                        }
                         // .sync.aligned: every lane of the warp, outside the row_ok branch
                         tc::tmem_st16(tmem + tl + (uint32_t)(2 * NH + col), fv);
                         tc::tmem_wait_st();
+                        if (m >= win0 && !in_win)
+                            win_plain_tmem(a.w + (size_t)(n0 + col) * a.Npad + row, a.Npad,
+                                           tmem + tl + (uint32_t)(2 * NH + col), row_ok);
                         if constexpr (TS) {
                             tc::fence_proxy_async_smem();
                             tc::named_bar(2 + csel, 128);
@@ -662,10 +680,15 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
                                     nb[ob + 2 * a.Npad] = cvt16<F16>(fs - from16<F16>(hi));
                                 }
                                 if (in_win) win_add(a.w + (size_t)(n0 + col + j) * a.Npad + row, fn);
-                                phl[j] = fn;
                             }
-                            if (plain_win)
-                                hqa_win_plain16(a.w + (size_t)(n0 + col) * a.Npad + row, a.Npad, phl);
+                            if (m >= win0 && !in_win) {
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) {
+                                    asm volatile("ld.shared.f32 %0, [%1];"
+                                                 : "=f"(phl[j]) : "r"(phis + (uint32_t)(col + j) * 512u + rloc * 4u));
+                                    win_plain(a.w + (size_t)(n0 + col + j) * a.Npad + row, phl[j]);
+                                }
+                            }
                         }
                         // .sync.aligned: every lane of the warp, outside the row_ok branch
                         tc::tmem_st16(tmem + tl + (uint32_t)(2 * NH + col), pv);
@@ -714,10 +737,14 @@ k_dense_md(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUte
                                     nb[ob + 2 * a.Npad] = cvt16<F16>(fs - from16<F16>(hi));
                                 }
                                 if (in_win) win_add(a.w + o, fn);
-                                ph[j] = fn;
                             }
-                            if (plain_win)
-                                hqa_win_plain16(a.w + (size_t)rbase * a.Npad + row, a.Npad, ph);
+                            if (m >= win0 && !in_win) {
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) {
+                                    const size_t o = (size_t)(rbase + j) * a.Npad + row;
+                                    win_plain(a.w + o, *(volatile float*)(a.phi + o));
+                                }
+                            }
                         }
                         if (more) {
 #pragma unroll

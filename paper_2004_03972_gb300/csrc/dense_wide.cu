@@ -75,6 +75,7 @@ k_dense_wide(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CU
     const uint32_t accf0 = bar + 24 * STAGES, acce0 = accf0 + 16, tmem_slot = accf0 + 32,
                    done_bar = accf0 + 40;
     __shared__ int s_abort;
+    __shared__ uint32_t s_tiny;   // *a.tiny: here, as a register held through the steps costs up to 3 %
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t crank = tc::cluster_rank();
     const int64_t U = (int64_t)w.RT * w.CB, total = U * a.S;
@@ -82,6 +83,7 @@ k_dense_wide(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CU
 
     if (threadIdx.x == 0) {
         s_abort = 0;
+        s_tiny = __ldcg(a.tiny);
         for (int s = 0; s < STAGES; ++s) {
             tc::mbar_init(full0 + 8 * s, 1);
             tc::mbar_init(empty0 + 8 * s, 1);
@@ -227,7 +229,6 @@ k_dense_wide(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CU
         const uint32_t acce_to = crank != 0 ? tc::mapa(acce0, 0) : acce0;
         const int mhalf = (a.M - 2) / 2;
         const int64_t win0 = a.S - (int64_t)a.W;
-        const bool tiny = __ldcg(a.tiny) != 0u;
         const int Kb = KSEG * a.Npad;         // operand row: [hi], [hi | lo] or [hi | hi | lo]
         bool stop = false;
         uint32_t i = 0;
@@ -236,7 +237,7 @@ k_dense_wide(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CU
             const int u = (int)(g % U), cb = u / w.RT, rt = u % w.RT;
             const uint32_t b = i & 1u;
             const float4 cf = __ldg(reinterpret_cast<const float4*>(a.sched) + m);
-            const bool in_win = m >= win0 && !tiny, plain_win = m >= win0 && tiny;
+            const bool in_win = m >= win0 && *(volatile uint32_t*)&s_tiny == 0u;
             const int row = rt * 2 * BM + (int)crank * BM + 32 * quarter + lane;
             const bool row_ok = row < a.N;
             const float hr = (a.h && row_ok) ? 2.f * __ldg(a.h + row) : 0.f;
@@ -289,9 +290,14 @@ k_dense_wide(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CU
                                 nb[ob + 2 * a.Npad] = cvt16<F16>(fs - from16<F16>(hi));
                             }
                             if (in_win) win_add(a.w + o, fn);
-                            ph[j] = fn;
                         }
-                        if (plain_win) hqa_win_plain16(a.w + (size_t)rbase * a.Npad + row, a.Npad, ph);
+                        if (m >= win0 && !in_win) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                const size_t o = (size_t)(rbase + j) * a.Npad + row;
+                                win_plain(a.w + o, *(volatile float*)(a.phi + o));
+                            }
+                        }
                     }
                     if (more) {
 #pragma unroll

@@ -57,16 +57,6 @@ __device__ __forceinline__ bool hqa_tiny_state(float phi, float p)
     return fabsf(phi) < 0x1p-80f && fabsf(p) < 0x1p-80f;
 }
 
-// 16 window sums without reductions: volatile, so past L1, one after another.
-__device__ __forceinline__ void hqa_win_plain16(float* w, size_t stride, const float (&v)[16])
-{
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        volatile float* o = w + j * stride;
-        *o = *o + v[j];
-    }
-}
-
 // One step of the kick/drift coefficient table (see hqa_run).
 struct StepCoef {
     float kA;  // c_j h alpha(j dt) M       multiplies phi^(M-1)
@@ -234,7 +224,7 @@ struct hqa_ctx {
     void* d_Jhcat = nullptr;       // [Mpad][3 Mpad] FP16 (J not exact in FP16 only)
     CUtensorMap tmJh;
     CUtensorMap tmJh3;
-    // plain FP32 dense path (CUDA cores): J in FP32, [Npad32][Npad32], built on first use
+    // FP32 dense fields, and runs of N > 19456 (CUDA cores): J in FP32, [Npad32][Npad32], built on first use
     float* d_Jf32 = nullptr;
     int Npad32 = 0;
     // FP32 dense path on the tensor cores: BF16 slices of J ([Mpad][3 Mpad], the
@@ -342,7 +332,7 @@ hqa_status hqa_dense_launch_md(hqa_ctx* ctx, const StepCoef* d_sched, int64_t S,
 // tensor map of a 16-bit [rows][cols] array (cols contiguous)
 bool hqa_dense_tmap16(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols,
                       uint32_t box_cols, uint32_t box_rows, bool swizzle, bool f16);
-// dense_f32.cu: the FP32 dense path on the tensor cores (fixed-point slices)
+// dense_f32.cu: FP32 dense runs on the tensor cores (BF16 slices)
 bool hqa_f32tc_possible(const hqa_ctx* ctx);
 hqa_status hqa_f32tc_prepare(hqa_ctx* ctx);
 void hqa_f32tc_plan(hqa_ctx* ctx, int32_t R, int* rb, int* grid, int* chunks);
@@ -350,7 +340,7 @@ hqa_status hqa_f32tc_launch_md(hqa_ctx* ctx, const StepCoef* d_sched, int64_t S,
                                int32_t R, uint64_t seed, int init, const float* phi0,
                                const float* p0, int M, float* phi_out, float* p_out,
                                float* phibar_out, cudaStream_t st);
-// dense_simt.cu: the plain FP32 dense path on the CUDA cores
+// dense_simt.cu: FP32 dense fields and the runs dense_f32.cu cannot take, on the CUDA cores
 bool hqa_simt_possible(const hqa_ctx* ctx);
 hqa_status hqa_simt_prepare(hqa_ctx* ctx);
 hqa_status hqa_simt_field(hqa_ctx* ctx, int32_t R, const float* phi, float* L, cudaStream_t st);
