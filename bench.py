@@ -313,7 +313,7 @@ def kernel_name(hqa, plan, prec_name):
     k = plan["kernel"]
     if k == hqa.KERNEL_DENSE:
         if prec_name == "PREC_FP32":
-            # 256 threads: the CUDA-core form; else the fixed-point slices on the tensor cores
+            # 256 threads: the CUDA-core form; else BF16 slices on the tensor cores
             return "k_dense_simt<1>" if plan.get("threads", 256) == 256 else "k_dense_f32"
         if plan.get("threads") == 320:
             return "k_dense_wide"

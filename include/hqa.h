@@ -85,8 +85,15 @@ enum {
 
 /* Arithmetic of the local-field operand.  phi and p stay FP32 in every case. */
 enum {
-    HQA_PREC_FP32 = 0,   /* phi operand FP32, FP32 accumulate (sparse kernels; dense
-                            contexts with HQA_KERNEL_DENSE: an FP32 GEMM on the CUDA cores) */
+    HQA_PREC_FP32 = 0,   /* phi operand FP32, FP32 accumulate (sparse kernels).  Dense
+                            contexts with HQA_KERNEL_DENSE: runs multiply phi (and real
+                            J) as three BF16 slices, 24 significant bits of every flux of
+                            ordinary size among its 32 neighbours in spin order, FP32
+                            accumulate, at an error below that of an FP32 sum unless such
+                            groups of one replica differ by 2^6 or more in scale (then up
+                            to N / 16 units of the last place of the partial sums); an
+                            FP32 GEMM on the CUDA cores for N > 19456 and for one-shot
+                            fields (hqa_local_field) */
     HQA_PREC_BF16 = 1,   /* phi operand rounded to BF16 (8 significant bits), FP32
                             accumulate; dense: J rounded to BF16 too (exact for +-1) */
     HQA_PREC_BF16X2 = 2, /* dense tensor-core path only: phi = hi + lo, both BF16 (about 16
@@ -109,16 +116,15 @@ enum {
                               accepted as stated where hqa_autotune chose it for the
                               context, replica count and precision */
     HQA_KERNEL_DENSE = 3,  /* dense contexts: the field as a GEMM of J and the replicas'
-                              fluxes -- on the tcgen05 tensor cores for the 16-bit
-                              precisions (BF16, BF16X2, FP16, FP16X2), on the CUDA cores
-                              for FP32 */
+                              fluxes on the tcgen05 tensor cores (see the precisions) */
     HQA_KERNEL_LOWDEG = 4, /* batch contexts whose members have at most 4 couplings per
                               spin and fewer than 2^15 spins: compact lists, operand and
                               state of a work item all in shared memory; replicas_per_block
                               1, 2 or 4.  AUTO picks it for such batches */
     HQA_KERNEL_STREAM = 5  /* single contexts with couplings in {-1, 0, +1}, FP32 or BF16:
-                              the operand and state in global memory (L2-resident at the
-                              sizes it serves), one persistent cooperative grid with a
+                              the operand in global memory (L2-resident at the sizes it
+                              serves), the rest of the state in its owner's shared memory
+                              as far as it fits, one persistent cooperative grid with a
                               bounded-wait barrier per step.  For instances whose operand
                               does not fit in one SM's shared memory; AUTO takes it when
                               the resident kernels cannot run (HQA_ERR_TOO_LARGE) or the
@@ -196,8 +202,8 @@ enum {
  * FP16X2 split phi into hi + lo and, when J is not exact in the format
  * (real-valued couplings), J as well: J_hi phi_hi + J_lo phi_hi +
  * J_hi phi_lo, about 16 (BF16) or 22 (FP16) significant bits of each.  FP32
- * with HQA_KERNEL_DENSE is an FP32 GEMM on the CUDA cores (any real J); FP32
- * with the sparse kernels needs couplings in {-1, 0, +1}.
+ * with HQA_KERNEL_DENSE takes any real J (held to 2^-25 of its row's largest);
+ * FP32 with the sparse kernels needs couplings in {-1, 0, +1}.
  * Errors: INVALID_ARG (N out of range, null J/out, unknown flag), ASYMMETRIC,
  * NONFINITE_INPUT, UNSUPPORTED (HQA_J_FP8), OOM, CUDA. */
 hqa_status hqa_create_dense(int32_t N, const float* J, const float* h, uint32_t flags,
@@ -273,9 +279,11 @@ hqa_status hqa_run(hqa_ctx* ctx, const hqa_schedule* sched, double dt, int64_t s
 
 /* Local field of the paper's kick (Methods, "Leapfrog algorithm"):
  *   L_i = sum_{j != i} J_ij phi_j + 2 h_i |phi_i|
- * for R replicas.  phi, L: device [R][N] float.  The sum is evaluated by
- * the same device code hqa_run would use with the same `opts` (precision,
- * replicas_per_block, kernel; NULL = defaults; init fields are ignored). */
+ * for R replicas.  phi, L: device [R][N] float.  The sum is evaluated at the
+ * precision and with the kernel and replica blocking that `opts` names (NULL =
+ * defaults; init fields are ignored), by the code hqa_run uses but for two forms
+ * that runs alone have: the FP32 slices of dense contexts (fields: an FP32 GEMM)
+ * and the small complete graphs of open options (fields: the list kernels). */
 hqa_status hqa_local_field(hqa_ctx* ctx, int32_t replicas, const float* phi, float* L,
                            const hqa_run_opts* opts, void* stream);
 
@@ -379,7 +387,7 @@ hqa_status hqa_solve_sub_noalloc(hqa_ctx* ctx, int32_t replicas, const int8_t* s
  * coupling entry (padding), shared-memory wavefronts per conflict-free
  * wavefront (bank conflicts), and mean/max warp load (balance). */
 typedef struct {
-    int32_t kernel;              /* HQA_KERNEL_SCALAR, _VECTOR or _DENSE */
+    int32_t kernel;              /* HQA_KERNEL_SCALAR, _VECTOR, _DENSE or _STREAM */
     int32_t replicas_per_block;
     int32_t blocks;              /* CTAs per launch */
     int32_t threads;             /* threads per CTA */

@@ -716,7 +716,7 @@ static hqa_status run_impl(hqa_ctx* ctx, const hqa_schedule* sched, double dt, i
     if (want_energy && !ctx->integer) return HQA_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (o.kernel == HQA_KERNEL_LOWDEG) return HQA_ERR_UNSUPPORTED;   // batch contexts only
-    int dense = 0;   // 1: tcgen05 GEMM, 2: FP32 CUDA-core GEMM
+    int dense = 0;   // as pick_dense
     s = pick_dense(ctx, replicas, o, &dense);
     if (s != HQA_OK) return s;
 
