@@ -275,11 +275,19 @@ __host__ __device__ inline int64_t first_cell(int64_t cells, int nv, int64_t b, 
     return cells / cell_unit(nv) * b / g * cell_unit(nv);
 }
 
+// Whether the lanes of a warp meet after their sums.  Where they lie in two rows or
+// more the sums end at different passes, and the lanes then stay apart up to the
+// barrier: FP32, N = 40000 x 100 21.9 -> 16.1 us a step, 20000 x 200 16.2 -> 15.2.
+// Rows of whole warps (N = 8000 x 128 6.0 / 6.4), rows of a few vectors (5000 x 8 3.4 /
+// 3.7, so many rows that some lane is always late) and BF16 (3 %) lose by it.
+inline bool lanes_meet(int nv, bool bf16) { return !bf16 && nv % 32 != 0 && nv >= 8; }
+
 // 16-byte state vectors of a cell: p, and in BF16 the FP32 master before it.
 template <bool BF16>
 constexpr int kPlanes = BF16 ? 4 : 1;
 
-template <bool BF16, bool STAGED>
+// MEET: the lanes of a warp come together after their sums (lanes_meet).
+template <bool BF16, bool STAGED, bool MEET>
 __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArgs a)
 {
     constexpr int V = Vec<BF16>::V, NP = kPlanes<BF16>;
@@ -323,9 +331,9 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
         void* nxt = (m & 1) ? a.op0 : a.op1;
         const bool in_win = m >= win0;
         int i = i0, v = v0;
-        // FP32: all lanes of a warp take part in every round, see below
-        for (int l = threadIdx.x; (BF16 ? l : l - (int)threadIdx.x) < mine; l += kMDThreads) {
-            const bool on = BF16 || l < mine;
+        // MEET: all lanes of a warp take part in each of its rounds
+        for (int l = threadIdx.x; (MEET ? l & ~31 : l) < mine; l += kMDThreads) {
+            const bool on = !MEET || l < mine;
             if (!on) {
                 i = rowA;
                 v = 0;
@@ -340,11 +348,7 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
                               [&](int k) { return s_ent[k]; }, L);
             else
                 cell_field<BF16>(a, cur, i, c, L);
-            // Where a warp's lanes lie in two rows or more, their sums end at different
-            // passes, and without this they stay apart up to the barrier: FP32, N =
-            // 40000 x 100 21.9 -> 16.1 us a step, 20000 x 200 16.2 -> 15.2.  In BF16 the
-            // same cost 3 %.
-            if constexpr (!BF16) __syncwarp();
+            if constexpr (MEET) __syncwarp();
             if (!on) break;
             const float hr = a.h ? 2.f * __ldg(a.h + i) : 0.f;
             const bool res = l < nres;
@@ -369,10 +373,11 @@ __global__ void __launch_bounds__(kMDThreads, 1) k_sparse_stream(const StreamArg
             // store's result without waiting for the load (bitwise outside the
             // states that hqa_tiny_state marks)
             if (in_win) {
+                const bool red = a.wred && s_tiny == 0u;
 #pragma unroll
                 for (int e = 0; e < V; e += 4) {
                     float4* w = reinterpret_cast<float4*>(a.w + o + e);
-                    if (a.wred && *(volatile uint32_t*)&s_tiny == 0u) {
+                    if (red) {
                         atomicAdd(w, make_float4(fn[e], fn[e + 1], fn[e + 2], fn[e + 3]));
                     } else {
                         float4 q = *w;
@@ -629,8 +634,9 @@ hqa_status hqa_stream_launch_md(hqa_ctx* ctx, int prec, const StepCoef* d_sched,
     // shares its memory with the resident state: rows that spread over more lines
     // (no whole warps) then gain more from L1.  us per step, all that fits resident /
     // this many: FP32 N = 60000 x 300 109 / 91, 60000 x 240 76 / 68; BF16 60000 x 400
-    // 122 / 103, 40000 x 400 70 / 65; rows of whole warps lost 5 %.
-    if (nv % 32 != 0 && touched(a.nres) > 0.8 * (double)ctx->l2_bytes)
+    // 122 / 103, 40000 x 400 70 / 65; nearer to L2 BF16 40000 x 300 (0.86 of L2) 45.8 /
+    // 47.7; rows of whole warps lost 5 %.
+    if (nv % 32 != 0 && touched(a.nres) > 0.9 * (double)ctx->l2_bytes)
         a.nres = std::min(a.nres, bf16 ? 1024 : 6144);
     const size_t smem = a.nres * cell_bytes + lists;
     // window sums by reductions while what a step touches in global memory (both
@@ -638,10 +644,13 @@ hqa_status hqa_stream_launch_md(hqa_ctx* ctx, int prec, const StepCoef* d_sched,
     // beyond, a reduction waits for its line from DRAM in L2 and holds up the
     // gathers (N = 40000 x 256 BF16, 100 steps: 5.5 ms without, 5.9 with)
     a.wred = touched(a.nres) + 4.0 * (double)n < 0.7 * (double)ctx->l2_bytes;
-    const void* fn = bf16 ? (staged ? (const void*)k_sparse_stream<true, true>
-                                    : (const void*)k_sparse_stream<true, false>)
-                          : (staged ? (const void*)k_sparse_stream<false, true>
-                                    : (const void*)k_sparse_stream<false, false>);
+    const bool meet = lanes_meet(nv, bf16);
+    const void* fn = bf16 ? (staged ? (const void*)k_sparse_stream<true, true, false>
+                                    : (const void*)k_sparse_stream<true, false, false>)
+                   : meet ? (staged ? (const void*)k_sparse_stream<false, true, true>
+                                    : (const void*)k_sparse_stream<false, false, true>)
+                          : (staged ? (const void*)k_sparse_stream<false, true, false>
+                                    : (const void*)k_sparse_stream<false, false, false>);
     if (hqa_smem_attr(fn, smem) != cudaSuccess) return HQA_ERR_CUDA;
     void* args[] = {&a};
     cudaLaunchAttribute attr[1];
