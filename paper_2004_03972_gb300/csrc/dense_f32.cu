@@ -465,9 +465,6 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                         // .sync.aligned: every lane of the warp, outside the row_ok branch
                         tc::tmem_st16(tl + PHI0 + (uint32_t)col, fv);
                         tc::tmem_wait_st();
-                        if (m >= win0 && !in_win)
-                            win_plain_tmem(a.w + (size_t)(n0 + col) * a.Npad + row, a.Npad,
-                                           tl + PHI0 + (uint32_t)col, row_ok);
                         tc::fence_proxy_async_smem();
                         tc::named_bar(2 + csel, 128);
                         if (gleader) {
@@ -506,6 +503,14 @@ k_dense_f32(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUt
                     atomicAdd(a.gbar + HV * nc + hh, 1u);
                 }
             }
+            // a marked state: the step's window sums, from the fluxes in TMEM
+            if (m >= win0 && !in_win && !stop)
+                for (int hh = 0; hh < HV; ++hh)
+                    for (int c = csel; c < NC / 16; c += kGroups) {
+                        const int col = hh * NC + c * 16;
+                        win_plain_tmem(a.w + (size_t)(n0 + col) * a.Npad + row, a.Npad,
+                                       tl + PHI0 + (uint32_t)col, row_ok);
+                    }
         }
         // final phi for the output kernel (p is already in global memory)
         for (int hh = 0; hh < HV; ++hh)

@@ -291,13 +291,6 @@ k_dense_wide(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CU
                             }
                             if (in_win) win_add(a.w + o, fn);
                         }
-                        if (m >= win0 && !in_win) {
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) {
-                                const size_t o = (size_t)(rbase + j) * a.Npad + row;
-                                win_plain(a.w + o, *(volatile float*)(a.phi + o));
-                            }
-                        }
                     }
                     if (more) {
 #pragma unroll
@@ -314,6 +307,15 @@ k_dense_wide(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CU
                     if (crank != 0) tc::mbar_arrive_remote(acce_to + 8 * b);
                     else tc::mbar_arrive(acce0 + 8 * b);
                 }
+                // a marked state: the unit's window sums, before another pair may have it
+                if (m >= win0 && !in_win && row_ok)
+#pragma unroll 1
+                    for (int c = csel; c < kNU / 16; c += kCS)
+#pragma unroll 1
+                        for (int j = 0; j < 16; ++j) {
+                            const size_t o = (size_t)(cb * kNU + c * 16 + j) * a.Npad + row;
+                            win_plain(a.w + o, *(volatile float*)(a.phi + o));
+                        }
             }
             // operand and state -> visible to the other CTAs' TMA loads and reads
             tc::fence_proxy_async_global();

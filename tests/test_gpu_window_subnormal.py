@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("kernel,prec_name,N,R", [
     ("KERNEL_DENSE", "PREC_FP32", 200, 40), ("KERNEL_DENSE", "PREC_BF16", 200, 40),
     ("KERNEL_DENSE", "PREC_FP16X2", 300, 70), ("KERNEL_DENSE", "PREC_BF16", 4993, 1030),
+    ("KERNEL_DENSE", "PREC_BF16", 2500, 2200),
     ("KERNEL_STREAM", "PREC_FP32", 700, 33), ("KERNEL_STREAM", "PREC_BF16", 700, 33)])
 def test_means_of_tiny_fluxes(kernel, prec_name, N, R):
     import torch
